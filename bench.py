@@ -46,7 +46,8 @@ def alg_bytes(prec):
 def kernel_bytes(kname, prec):
     """Bytes per site that a lattice kernel itself must move (arrays touched
     once): the density pass reads the populations and the mask and writes
-    rho^k and j^A + j^B; the lean momentum kernel reads j^A + j^B, psi^k and
+    rho^k and j^A + j^B; the moment kernel reads and writes rho^k and j and
+    reads the 4-byte link classes; the lean momentum kernel reads j^A + j^B, psi^k and
     the 4-byte link classes and writes the populations; the two-pass kernel
     reads both; the plain kernel reads and writes the populations."""
     pops = 38 * STORE[prec]
@@ -54,6 +55,8 @@ def kernel_bytes(kname, prec):
         return pops + 1 + 5 * COMPUTE[prec]
     if kname == "k_lean":
         return pops + 5 * COMPUTE[prec] + 4
+    if kname == "k_moments":
+        return 10 * COMPUTE[prec] + 4
     if kname == "k_fused_async":
         return 2 * pops + 2 * COMPUTE[prec] + 4
     return 2 * pops + 1
@@ -467,20 +470,22 @@ def main():
     kname = lat.fused_kernel()
     abytes = alg_bytes(args.prec)
     alg = abytes * w.n_sites
+    # per step: at tau = 1 the steps of a call between the first and the last
+    # run from moments to moments, and the density pass runs once a call
     kavg = kern_ms / max(kern_n, 1)
-    davg = dens_ms / dens_n if dens_n else 0.0
+    davg = dens_ms / max(kern_n, 1)
     traffic = recorded_traffic(args.prec)
-    # The lattice update of a time step (one read and one write of every
-    # population: the method's algorithmic bytes) is done by the density pass
-    # and the lean kernel (with its small wall kernel) together when
-    # particles are present, by the fused kernel alone otherwise; frac is
-    # their rate against the measured copy bandwidth, step_frac the same
-    # bytes over the whole step.
+    # frac is the rate of the lattice kernels against the measured copy
+    # bandwidth for one read and one write of every population a step (the
+    # bytes of a step that keeps its state in populations: above 1 where the
+    # steps of a call keep rho^k and j instead, whose own bytes are in
+    # `kernels`); step_frac the same bytes over the whole step.
     lattice_ms = kavg + davg
     achieved = alg / (lattice_ms / 1e3) / 1e9
-    kernels = [{"kernel": kname, "ms": round(kavg, 4), "own_bytes_per_site": kernel_bytes(kname, args.prec),
-                "own_frac": round(kernel_bytes(kname, args.prec) * w.n_sites / (kavg / 1e3) / 1e9 / peak, 4)}]
-    if dens_n:
+    steps_kname = "k_moments" if dens_n < kern_n and kname == "k_lean" else kname
+    kernels = [{"kernel": steps_kname, "ms": round(kavg, 4), "own_bytes_per_site": kernel_bytes(steps_kname, args.prec),
+                "own_frac": round(kernel_bytes(steps_kname, args.prec) * w.n_sites / (kavg / 1e3) / 1e9 / peak, 4)}]
+    if dens_n == kern_n:
         kernels.insert(0, {"kernel": "k_density", "ms": round(davg, 4),
                            "own_bytes_per_site": kernel_bytes("k_density", args.prec),
                            "own_frac": round(kernel_bytes("k_density", args.prec) * w.n_sites / (davg / 1e3) / 1e9
@@ -543,7 +548,7 @@ def main():
             m2 = max_over_ranks(time_steps(L2, steps, torch), world, dev)
             km, kn = L2.profile_read()
             dm, dn = L2.profile_read(LB_KERNEL_DENSITY)
-            kk = km / max(kn, 1) + (dm / dn if dn else 0.0)
+            kk = (km + dm) / max(kn, 1)
             forms[prec] = {"mlups": round(world * N * steps / (m2 / 1e3) / 1e6, 1), "steps": steps,
                            "kernel": L2.fused_kernel(),
                            "kernel_frac": round(alg_bytes(prec) * N / (kk / 1e3) / 1e9 / peak, 4),

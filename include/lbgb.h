@@ -161,7 +161,12 @@ int lb_add_colloids(lb_ctx *ctx, int n, const double *pos, const double *vel,
                     const double *omega, const double *quat, const double *radius,
                     const double *mass);
 
-/* Advance nsteps time steps.  Returns LB_ERR_NONFINITE / LB_ERR_OVERLAP if the
+/* Advance nsteps time steps.  The state a call leaves is the populations
+ * f(t + nsteps).  At tau_A = tau_B = 1 (FP32 and FP16 contexts, no recording,
+ * no LB_ROUND_NEAREST) a call of several steps keeps rho^k and j in FP32
+ * between them, which is all that Eq. 16 needs at omega = 1, so that only the
+ * first step reads and only the last one stores populations: a run split
+ * into other calls differs by rounding.  Returns LB_ERR_NONFINITE / LB_ERR_OVERLAP if the
  * device flagged the condition during these steps (state then undefined). */
 int lb_step(lb_ctx *ctx, int nsteps);
 
@@ -196,7 +201,8 @@ int lb_get_owner(lb_ctx *ctx, int *out);
 /* Kernel timing.  While enabled, lb_step records a CUDA event pair on the
  * context stream around every launch of the fused lattice kernel (the
  * collide + Shan-Chen + stream + bounce-back kernel, the dominant one, with
- * the small wall kernel that follows it in the lean form; LB_KERNEL_FUSED)
+ * the small wall kernel that follows it in the lean form, or the kernels of a
+ * step from moments to moments; LB_KERNEL_FUSED)
  * and around the full density pass that precedes it when particles are
  * present (LB_KERNEL_DENSITY; see lb_fused_kernel).
  * lb_profile(ctx, 1) enables and clears the records, lb_profile(ctx, 0)
@@ -331,7 +337,9 @@ long long lb_pair_list_builds(lb_ctx *ctx);
  *      moments (Eq. 16 at omega = 1), staging the halo of rho^k in shared
  *      memory with asynchronous copies, pushes the links and bounces those
  *      into particle nodes (Eqs. 17-19, 22, 23); a small kernel then applies
- *      the rules of the z faces (Eqs. 9, 10);
+ *      the rules of the z faces (Eqs. 9, 10).  Of a call of several steps
+ *      (see lb_step) the density pass belongs to the first one and the lean
+ *      kernel to the last one, with a kernel from moments to moments between;
  *  LB_FUSED_TWO_PASS  particles, other tau: a density pass writes rho^k, the
  *      fused kernel re-reads the populations;
  *  LB_FUSED_PLAIN     no particles, other tau: one pass, halo densities

@@ -387,6 +387,14 @@ int lb_init_fields(lb_ctx* ctx, const double* rhoA, const double* rhoB, const do
     if (L.ncomp == 2) CK(cudaMemcpyAsync(st + L.N, rhoB, nb, cudaMemcpyHostToDevice, ctx->stream), "copy rhoB");
     if (u) CK(cudaMemcpyAsync(st + 2 * L.N, u, 3 * nb, cudaMemcpyHostToDevice, ctx->stream), "copy u");
     else CK(cudaMemsetAsync(st + 2 * L.N, 0, 3 * nb, ctx->stream), "zero u");
+    // any density near those of the fluid serves: the mean of some sites
+    const double* rho[2] = {rhoA, rhoB};
+    for (int k = 0; k < L.ncomp; k++) {
+        double sum = 0.0;
+        const long long step = L.N / 1024 + 1, n = (L.N + step - 1) / step;
+        for (long long s = 0; s < L.N; s += step) sum += rho[k][s];
+        L.rref[k] = isfinite((float)(sum / n)) ? (float)(sum / n) : 0.f;
+    }
     L.nc = 0;
     ctx->all_fixed = 1;
     ctx->sr_step = 0;  // a new state starts the rounding sequence afresh
@@ -510,23 +518,91 @@ static int ensure_link_classes(lb_ctx* ctx, cudaStream_t st) {
     return launch_link_classes(ctx->L, true, st);
 }
 
+// A call of several steps at tau = 1 keeps rho^k and j between its steps
+// instead of the populations (lbgb_moment.cu): the first step takes them from
+// the populations, the last one pushes the populations.  While it runs the
+// populations f(t) are dead after the first density pass, so their buffer
+// holds the second copy of the moments.  Recording needs the populations of
+// every step, and LB_ROUND_NEAREST asks for their rounding in every step.
+struct MomentRun {
+    bool on;
+    void *psi[2], *mom[2];  // the moments of time t and the place of those of t + 1
+};
+
+static MomentRun moment_run(const lb_ctx* ctx, int nsteps) {
+    const Lattice& L = ctx->L;
+    MomentRun m;
+    m.on = nsteps > 1 && L.P.tau[0] == 1.0 && (L.ncomp == 1 || L.P.tau[1] == 1.0) && ctx->rec_left <= 0 && ctx->prec != LB_FP64 &&
+           (ctx->prec != LB_FP16 || L.sr);
+    const size_t c = compute_bytes(ctx->prec);
+    const size_t rho = align_up((size_t)L.ncomp * L.N * c), all = rho + align_up((size_t)3 * L.pstride * c);
+    char* cur = (char*)L.f_cur;
+    if (L.ncomp == 2) {
+        m.psi[0] = L.psi;
+        m.mom[0] = L.mom;
+        m.psi[1] = cur;
+        m.mom[1] = cur + rho;
+    } else {
+        // the one-component lattice has no arrays for them: from the second
+        // buffer (the density pass) to two places in the first one
+        m.psi[0] = L.f_nxt;
+        m.mom[0] = (char*)L.f_nxt + rho;
+        m.psi[1] = cur;
+        m.mom[1] = cur + rho;
+    }
+    // (19 ncomp populations a site are larger than two, or for two
+    // components one, set of ncomp + 3 values of the compute type)
+    if ((L.ncomp == 2 ? all : 2 * all) > state_bytes(ctx)) m.on = false;
+    return m;
+}
+
 int lb_step(lb_ctx* ctx, int nsteps) {
     if (!ctx || nsteps < 0) return LB_ERR_ARG;
     if (!ctx->have_fields) return set_err(ctx, LB_ERR_STATE, "lb_init_fields must come first");
     Lattice& L = ctx->L;
     cudaStream_t s = ctx->stream;
     CK(cudaMemsetAsync(L.flags, 0, 4, s), "clear flags");
+    MomentRun run = moment_run(ctx, nsteps);
+    Lattice V = L;  // the view the kernels get: psi and mom of the present time
     for (int t = 0; L.ncomp == 1 && t < nsteps; t++) {
         // the one-component fluid: one kernel per step (Eqs. 5-7, 16, 3, 9)
         if (L.sr) L.sr_key = sr_key(ctx->sr_seed, ctx->sr_step++);
-        const int n0 = launch_single_face_values(L, ctx->prec, s);  // extrapolated face densities
+        const bool last = !run.on || t == nsteps - 1;
+        V.f_cur = L.f_cur;
+        V.f_nxt = L.f_nxt;
+        V.sr_key = L.sr_key;
+        int n = 0;
+        if (run.on) {
+            V.psi = run.psi[0];
+            V.mom = run.mom[0];
+            if (t == 0) {
+                if (int rc = prof_mark(ctx, LB_KERNEL_DENSITY, 0, s)) return rc;
+                n += launch_single_moments(V, ctx->prec, s);
+                if (int rc = prof_mark(ctx, LB_KERNEL_DENSITY, 1, s)) return rc;
+            }
+        }
+        n += launch_single_face_values(V, ctx->prec, run.on, s);  // extrapolated face densities
         if (int rc = prof_mark(ctx, LB_KERNEL_FUSED, 0, s)) return rc;
-        const int n = n0 + launch_single_step(L, ctx->prec, s);
+        if (!last) n += launch_moments(V, run.psi[1], run.mom[1], s);
+        else n += run.on ? launch_single_push(V, ctx->prec, s) : launch_single_step(V, ctx->prec, s);
         if (int rc = prof_mark(ctx, LB_KERNEL_FUSED, 1, s)) return rc;
         if (int rc = launched(ctx, n, "step kernel")) return rc;
-        void* tmp = L.f_cur;
-        L.f_cur = L.f_nxt;
-        L.f_nxt = tmp;
+        if (last) {
+            void* tmp = L.f_cur;
+            L.f_cur = L.f_nxt;
+            L.f_nxt = tmp;
+        } else {
+            // the place the moments were in is free now; after the first
+            // step it is the other half of the first buffer, because the
+            // second one receives the populations
+            const size_t all = (char*)run.mom[1] - (char*)run.psi[1] + align_up((size_t)3 * L.pstride * compute_bytes(ctx->prec));
+            void* p = t == 0 ? (char*)run.psi[1] + all : run.psi[0];
+            void* m = t == 0 ? (char*)run.mom[1] + all : run.mom[0];
+            run.psi[0] = run.psi[1];
+            run.mom[0] = run.mom[1];
+            run.psi[1] = p;
+            run.mom[1] = m;
+        }
         ctx->stepped = 1;
     }
     for (int t = 0; L.ncomp == 2 && t < nsteps; t++) {
@@ -544,14 +620,7 @@ int lb_step(lb_ctx* ctx, int nsteps) {
             CK(cudaEventRecord(ctx->ev_join, ctx->side), "join event");
         }
         if (L.sr) L.sr_key = sr_key(ctx->sr_seed, ctx->sr_step++);
-        n += launch_remap(L, ctx->prec, ctx->maxc, s);  // destroy / create (Eqs. 24, 25)
         const bool unit = L.P.tau[0] == 1.0 && L.P.tau[1] == 1.0;
-        if (L.nc > 0) {
-            n += launch_link_classes(L, !ctx->nb_valid, s);
-            ctx->nb_valid = 1;
-        } else if (unit) {
-            n += ensure_link_classes(ctx, s);  // no particles: every word 0, once
-        }
         // rho^k (Eq. 6) of every fluid node when particles need virtual
         // densities (Eq. 20) or omega = 1; with omega = 1 the pass also
         // writes j^k, and the lean kernel collides from the moments instead of
@@ -560,27 +629,48 @@ int lb_step(lb_ctx* ctx, int nsteps) {
         // its halo densities itself).
         L.dense_psi = L.nc > 0 || unit;
         L.dense_mom = L.dense_psi && unit;
-        if (L.dense_psi) {
-            if (int rc = prof_mark(ctx, LB_KERNEL_DENSITY, 0, s)) return rc;
-            n += launch_density(L, ctx->prec, s);
-            if (int rc = prof_mark(ctx, LB_KERNEL_DENSITY, 1, s)) return rc;
-        } else {
-            n += launch_shell_density(L, ctx->prec, s);
+        const bool last = !run.on || t == nsteps - 1, kept = run.on && t > 0;
+        V = L;
+        if (run.on) {
+            V.psi = run.psi[0];
+            V.mom = run.mom[0];
         }
-        n += launch_wall_psi(L, ctx->prec, s);         // wall densities
-        n += launch_face_values(L, ctx->prec, s);      // extrapolated open-face values (Sec. 2.2)
-        n += launch_virtual(L, ctx->prec, 1, s);       // Eqs. 20, 21
+        n += launch_remap(V, ctx->prec, ctx->maxc, kept, s);  // destroy / create (Eqs. 24, 25)
+        if (L.nc > 0) {
+            n += launch_link_classes(V, !ctx->nb_valid, s);
+            ctx->nb_valid = 1;
+        } else if (unit) {
+            n += ensure_link_classes(ctx, s);  // no particles: every word 0, once
+        }
+        if (L.dense_psi && !kept) {
+            if (int rc = prof_mark(ctx, LB_KERNEL_DENSITY, 0, s)) return rc;
+            n += launch_density(V, ctx->prec, s);
+            if (int rc = prof_mark(ctx, LB_KERNEL_DENSITY, 1, s)) return rc;
+        } else if (!L.dense_psi) {
+            n += launch_shell_density(V, ctx->prec, s);
+        }
+        n += launch_wall_psi(V, ctx->prec, s);           // wall densities
+        n += launch_face_values(V, ctx->prec, kept, s);  // extrapolated open-face values (Sec. 2.2)
+        n += launch_virtual(V, ctx->prec, 1, s);         // Eqs. 20, 21
         if (int rc = prof_mark(ctx, LB_KERNEL_FUSED, 0, s)) return rc;
         // Eqs. 11, 14, 16, 3, 9, 17; the link forces of Eqs. 19, 22, 23
-        n += launch_fluid_step(L, ctx->prec, s);
+        n += last ? launch_fluid_step(V, ctx->prec, s) : launch_moments(V, run.psi[1], run.mom[1], s);
         if (int rc = prof_mark(ctx, LB_KERNEL_FUSED, 1, s)) return rc;
         if (L.nc > 0) CK(cudaStreamWaitEvent(s, ctx->ev_join, 0), "join wait");
         n += launch_integrate(L, s);  // Eqs. 28-35
         int rc = launched(ctx, n, "step kernels");
         if (rc) return rc;
-        void* tmp = L.f_cur;
-        L.f_cur = L.f_nxt;
-        L.f_nxt = tmp;
+        if (last) {
+            void* tmp = L.f_cur;
+            L.f_cur = L.f_nxt;
+            L.f_nxt = tmp;
+        } else {
+            for (void** p : {run.psi, run.mom}) {
+                void* tmp = p[0];
+                p[0] = p[1];
+                p[1] = tmp;
+            }
+        }
         ctx->stepped = 1;
         if (rec) {
             if (ctx->rec_forces && L.nc > 0)

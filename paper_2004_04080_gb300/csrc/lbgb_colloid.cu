@@ -300,6 +300,44 @@ __device__ __forceinline__ typename Prec<PREC>::C site_rho(const Lattice& L, lon
     return r;
 }
 
+// rho^k of a fluid node, from the populations or (MOM) from the moments
+template <int PREC, bool MOM>
+__device__ __forceinline__ typename Prec<PREC>::C node_rho(const Lattice& L, long long s, int k) {
+    typedef typename Prec<PREC>::C C;
+    if (MOM) return ((const C*)L.psi)[2 * s + k];
+    return site_rho<PREC>(L, s, k);
+}
+
+// the state of a node the particles release: f = f^eq(rb^k, uw), or (MOM) its
+// moments
+template <int PREC, bool MOM>
+__device__ __forceinline__ void store_refill(const Lattice& L, long long s, const typename Prec<PREC>::C (&rb)[2],
+                                             const typename Prec<PREC>::C (&uw)[3]) {
+    typedef typename Prec<PREC>::S S;
+    typedef typename Prec<PREC>::C C;
+    if (MOM) {
+        for (int k = 0; k < 2; k++) ((C*)L.psi)[2 * s + k] = rb[k];
+        for (int d = 0; d < 3; d++) ((C*)L.mom)[d * L.pstride + s] = (rb[0] + rb[1]) * uw[d];
+        return;
+    }
+    const C uu = uw[0] * uw[0] + uw[1] * uw[1] + uw[2] * uw[2];
+    S* f = (S*)L.f_cur;
+    for (int k = 0; k < 2; k++)
+        for (int i = 0; i < Q; i++)
+            st_pop(f + pop_index(k * Q + i, s, L.pstride), feq<C>(i, rb[k], uw[0], uw[1], uw[2], uu),
+                   pop_shift<S, C>(L, k, i));
+}
+
+// a node a particle covers holds no fluid (MOM: the density pass is not run again)
+template <int PREC, bool MOM>
+__device__ __forceinline__ void clear_moments(const Lattice& L, long long s) {
+    typedef typename Prec<PREC>::C C;
+    if (MOM) {
+        for (int k = 0; k < 2; k++) ((C*)L.psi)[2 * s + k] = C(0);
+        for (int d = 0; d < 3; d++) ((C*)L.mom)[d * L.pstride + s] = C(0);
+    }
+}
+
 // -------------------------------------------------- FP32 snapshot
 __global__ void k_snapshot(Lattice L) {
     int p = blockIdx.x * blockDim.x + threadIdx.x;
@@ -377,7 +415,7 @@ __device__ __forceinline__ void particle_frame(const Lattice& L, int p, int x, i
 // Classify the points around particle p at its new position r_p(t):
 //   fluid node now inside -> destroy (Eq. 24): its momentum rho u goes to p
 //   node of p now outside -> create (handled by k_remap_create)
-template <int PREC>
+template <int PREC, bool MOM>
 __global__ void __launch_bounds__(PB) k_remap_classify(Lattice L) {
     typedef typename Prec<PREC>::C C;
     int p = blockIdx.x;
@@ -396,11 +434,16 @@ __global__ void __launch_bounds__(PB) k_remap_classify(Lattice L) {
                     return;
                 }
                 list_changed(L, s);
-                C fv[2][Q], rho[2], j[2][3], u[3], om;
-                load_site<PREC>(L, (const typename Prec<PREC>::S*)L.f_cur, s, fv, rho, j);
-                mixture<C>(L, rho, j, u, om);
-                C rt = rho[0] + rho[1];
-                C mom[3] = {rt * u[0], rt * u[1], rt * u[2]}, tq[3];
+                C mom[3], tq[3];
+                if (MOM) {  // rho u = j at equal tau
+                    for (int m = 0; m < 3; m++) mom[m] = ((const C*)L.mom)[m * L.pstride + s];
+                } else {
+                    C fv[2][Q], rho[2], j[2][3], u[3], om;
+                    load_site<PREC>(L, (const typename Prec<PREC>::S*)L.f_cur, s, fv, rho, j);
+                    mixture<C>(L, rho, j, u, om);
+                    C rt = rho[0] + rho[1];
+                    for (int m = 0; m < 3; m++) mom[m] = rt * u[m];
+                }
                 crs<C>(d, mom, tq);
 #pragma unroll
                 for (int m = 0; m < 3; m++) {
@@ -427,9 +470,8 @@ __global__ void __launch_bounds__(PB) k_remap_classify(Lattice L) {
 // Refill the nodes released by p (Eq. 25): f = f^eq(rhobar^k, u_w) with
 // rhobar^k the w_i-weighted mean over neighbours that are fluid before and
 // after the remap, u_w = v_p + omega_p x (r - r_p); p loses (rhobar) u_w.
-template <int PREC>
+template <int PREC, bool MOM>
 __global__ void __launch_bounds__(PB) k_remap_create(Lattice L) {
-    typedef typename Prec<PREC>::S S;
     typedef typename Prec<PREC>::C C;
     if (*L.nb_chg <= NB_CHG_CAP) return;  // the list kernel does it
     int p = blockIdx.x;
@@ -447,8 +489,8 @@ __global__ void __launch_bounds__(PB) k_remap_create(Lattice L) {
             long long m = nbr_index(L, n, i);
             if (L.owner[m] != -1 || L.evt[m] != 0) continue;
             C w = wgt<C>(i);
-            num[0] += w * site_rho<PREC>(L, m, 0);
-            num[1] += w * site_rho<PREC>(L, m, 1);
+            num[0] += w * node_rho<PREC, MOM>(L, m, 0);
+            num[1] += w * node_rho<PREC, MOM>(L, m, 1);
             den += w;
         }
         C rb[2];
@@ -456,12 +498,7 @@ __global__ void __launch_bounds__(PB) k_remap_create(Lattice L) {
         C wxd[3], uw[3];
         crs<C>(g.w, d, wxd);
         for (int m = 0; m < 3; m++) uw[m] = g.v[m] + wxd[m];
-        C uu = uw[0] * uw[0] + uw[1] * uw[1] + uw[2] * uw[2];
-        S* f = (S*)L.f_cur;
-        for (int k = 0; k < 2; k++)
-            for (int i = 0; i < Q; i++)
-                st_pop(f + pop_index(k * Q + i, s, L.pstride), feq<C>(i, rb[k], uw[0], uw[1], uw[2], uu),
-                       pop_shift<S, C>(L, k, i));
+        store_refill<PREC, MOM>(L, s, rb, uw);
         C rt = rb[0] + rb[1];
         C mom[3] = {-rt * uw[0], -rt * uw[1], -rt * uw[2]}, tq[3];
         crs<C>(d, mom, tq);
@@ -481,7 +518,7 @@ __global__ void __launch_bounds__(PB) k_remap_create(Lattice L) {
 }
 
 // Commit the new node map of particle p.
-template <int PREC>
+template <int PREC, bool MOM>
 __global__ void __launch_bounds__(PB) k_remap_commit(Lattice L) {
     typedef typename Prec<PREC>::C C;
     if (*L.nb_chg <= NB_CHG_CAP) return;  // the list kernel does it
@@ -494,6 +531,7 @@ __global__ void __launch_bounds__(PB) k_remap_commit(Lattice L) {
             int old = atomicCAS(L.owner + s, -1, p);
             if (old != -1) atomicOr(L.flags, FLAG_OVERLAP);
             L.mask[s] = 1;
+            clear_moments<PREC, MOM>(L, s);
             L.evt[s] = 0;
         } else if (e == 4 * (p + 1) + 2) {
             L.owner[s] = -1;
@@ -507,9 +545,8 @@ __global__ void __launch_bounds__(PB) k_remap_commit(Lattice L) {
 // per listed node (k_remap_create's work when the list is complete): the
 // momentum (rhobar) u_w each one carries off its particle is added to F_c,
 // T_c as its own fixed-point term.
-template <int PREC>
+template <int PREC, bool MOM>
 __global__ void k_remap_create_list(Lattice L) {
-    typedef typename Prec<PREC>::S S;
     typedef typename Prec<PREC>::C C;
     const int cnt = *L.nb_chg;
     if (cnt > NB_CHG_CAP) return;
@@ -527,8 +564,8 @@ __global__ void k_remap_create_list(Lattice L) {
             long long m = nbr_index(L, n, i);
             if (L.owner[m] != -1 || L.evt[m] != 0) continue;
             C w = wgt<C>(i);
-            num[0] += w * site_rho<PREC>(L, m, 0);
-            num[1] += w * site_rho<PREC>(L, m, 1);
+            num[0] += w * node_rho<PREC, MOM>(L, m, 0);
+            num[1] += w * node_rho<PREC, MOM>(L, m, 1);
             den += w;
         }
         C rb[2];
@@ -537,12 +574,7 @@ __global__ void k_remap_create_list(Lattice L) {
         particle_frame<C>(L, p, X, Y, Z, d, v, w);
         crs<C>(w, d, wxd);
         for (int m = 0; m < 3; m++) uw[m] = v[m] + wxd[m];
-        C uu = uw[0] * uw[0] + uw[1] * uw[1] + uw[2] * uw[2];
-        S* f = (S*)L.f_cur;
-        for (int k = 0; k < 2; k++)
-            for (int i = 0; i < Q; i++)
-                st_pop(f + pop_index(k * Q + i, s, L.pstride), feq<C>(i, rb[k], uw[0], uw[1], uw[2], uu),
-                       pop_shift<S, C>(L, k, i));
+        store_refill<PREC, MOM>(L, s, rb, uw);
         C rt = rb[0] + rb[1];
         C mom[3] = {-rt * uw[0], -rt * uw[1], -rt * uw[2]}, tq[3];
         crs<C>(d, mom, tq);
@@ -554,6 +586,7 @@ __global__ void k_remap_create_list(Lattice L) {
 }
 
 // Commit the listed nodes (k_remap_commit's work when the list is complete).
+template <int PREC, bool MOM>
 __global__ void k_remap_commit_list(Lattice L) {
     const int cnt = *L.nb_chg;
     if (cnt > NB_CHG_CAP) return;
@@ -564,6 +597,7 @@ __global__ void k_remap_commit_list(Lattice L) {
             int old = atomicCAS(L.owner + s, -1, p);
             if (old != -1) atomicOr(L.flags, FLAG_OVERLAP);
             L.mask[s] = 1;
+            clear_moments<PREC, MOM>(L, s);
         } else if ((e & 3) == 2) {
             L.owner[s] = -1;
             L.mask[s] = 0;
@@ -1181,7 +1215,20 @@ int launch_map_initial(const Lattice& L, int prec, int first, int count, cudaStr
     return 1;
 }
 
-int launch_remap(const Lattice& L, int prec, int maxc, cudaStream_t st) {
+template <int P, bool MOM>
+static void launch_remap_t(const Lattice& L, cudaStream_t st) {
+    const dim3 grid((unsigned)L.nc, REMAP_GROUPS);
+    k_remap_classify<P, MOM><<<grid, PBLK, 0, st>>>(L);
+    // the refill and the commit of the listed nodes; the per-particle shell
+    // scans return at once unless the list overflowed
+    const unsigned lg = (unsigned)(2 * device_sms());
+    k_remap_create_list<P, MOM><<<lg, 128, 0, st>>>(L);
+    k_remap_create<P, MOM><<<grid, PBLK, 0, st>>>(L);
+    k_remap_commit_list<P, MOM><<<lg, 128, 0, st>>>(L);
+    k_remap_commit<P, MOM><<<grid, PBLK, 0, st>>>(L);
+}
+
+int launch_remap(const Lattice& L, int prec, int maxc, bool moments, cudaStream_t st) {
     if (L.nc <= 0) return 0;
     // the per-particle terms of the step are fixed-point sums of block
     // partials and per-site contributions (acc_add), from zero; the
@@ -1189,15 +1236,11 @@ int launch_remap(const Lattice& L, int prec, int maxc, cudaStream_t st) {
     (void)maxc;
     cudaMemsetAsync(L.acc, 0, (size_t)ACC_TERMS * L.maxc * 6 * sizeof(unsigned long long), st);
     cudaMemsetAsync(L.nb_chg, 0, sizeof(int), st);
-    const dim3 grid((unsigned)L.nc, REMAP_GROUPS);
-    DISPATCHC(prec, (k_remap_classify<P><<<grid, PBLK, 0, st>>>(L)));
-    // the refill and the commit of the listed nodes; the per-particle shell
-    // scans return at once unless the list overflowed
-    const unsigned lg = (unsigned)(2 * device_sms());
-    DISPATCHC(prec, (k_remap_create_list<P><<<lg, 128, 0, st>>>(L)));
-    DISPATCHC(prec, (k_remap_create<P><<<grid, PBLK, 0, st>>>(L)));
-    k_remap_commit_list<<<lg, 128, 0, st>>>(L);
-    DISPATCHC(prec, (k_remap_commit<P><<<grid, PBLK, 0, st>>>(L)));
+    if (moments) {
+        DISPATCHC(prec, (launch_remap_t<P, true>(L, st)));
+    } else {
+        DISPATCHC(prec, (launch_remap_t<P, false>(L, st)));
+    }
     return 5;
 }
 

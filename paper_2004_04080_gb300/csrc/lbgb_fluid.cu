@@ -114,10 +114,21 @@ __global__ void k_wall_psi(Lattice L) {
 }
 
 // rho^k and the mixture velocity u (Eqs. 6, 7, 14) of fluid node s from f(t)
-template <int PREC>
+// (MOM: from the moments of a run at tau = 1)
+template <int PREC, bool MOM>
 __device__ __forceinline__ void node_values(const Lattice& L, long long s, typename Prec<PREC>::C (&q)[5]) {
     typedef typename Prec<PREC>::S S;
     typedef typename Prec<PREC>::C C;
+    if (MOM) {
+        const C* psi = (const C*)L.psi;
+        const C* mom = (const C*)L.mom;
+        q[0] = psi[2 * s];
+        q[1] = psi[2 * s + 1];
+        const C ir = C(1) / (q[0] + q[1]);
+#pragma unroll
+        for (int d = 0; d < 3; d++) q[2 + d] = mom[d * L.pstride + s] * ir;
+        return;
+    }
     const S* f = (const S*)L.f_cur;
     C rho[2] = {0, 0}, j[2][3] = {{0, 0, 0}, {0, 0, 0}};
 #pragma unroll
@@ -147,7 +158,7 @@ __device__ __forceinline__ void node_values(const Lattice& L, long long s, typen
 // or nz < 2.  From f(t) after the remap, like every lattice kernel of the
 // step.  The face rules read rho_w of velocity faces (Eq. 9) and u_w of
 // pressure faces (Eq. 10) from here.
-template <int PREC>
+template <int PREC, bool MOM>
 __global__ void k_face_values(Lattice L) {
     typedef typename Prec<PREC>::C C;
     const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y, side = blockIdx.z;
@@ -158,30 +169,16 @@ __global__ void k_face_values(Lattice L) {
     const long long b = col + nxy * zb;
     if (L.mask[b]) return;  // a particle node on the face keeps what it holds
     C q[5];
-    node_values<PREC>(L, b, q);
+    node_values<PREC, MOM>(L, b, q);
     if (zi >= 0 && zi < L.nz && !L.mask[col + nxy * zi]) {
         C qi[5];
-        node_values<PREC>(L, col + nxy * zi, qi);
+        node_values<PREC, MOM>(L, col + nxy * zi, qi);
 #pragma unroll
         for (int a = 0; a < 5; a++) q[a] += C(0.5) * (q[a] - qi[a]);
     }
     C* fv = (C*)L.face + 5 * (side * nxy + col);
 #pragma unroll
     for (int a = 0; a < 5; a++) fv[a] = q[a];
-}
-
-// Add the link force and torque of one site (Eqs. 22, 23) to the fixed-point
-// sums of F_liq, T_liq of its particle (p < 0: no link of the site reaches a
-// particle).  Integer atomics: the sums do not depend on the order of the
-// additions, so they are the same bits on every run.
-template <typename C>
-__device__ __forceinline__ void commit_link_forces(const Lattice& L, int p, const C (&F)[3], const C (&T)[3]) {
-    if (p < 0) return;
-#pragma unroll
-    for (int d = 0; d < 3; d++) {
-        acc_add(L, acc_slot(L, ACC_FLIQ, p, d), F[d]);
-        acc_add(L, acc_slot(L, ACC_TLIQ, p, d), T[d]);
-    }
 }
 
 // ------------------------------------------------------- fused step
@@ -1441,11 +1438,15 @@ int launch_wall_bounce(const Lattice& L, int prec, cudaStream_t st) {
     return 1;
 }
 
-int launch_face_values(const Lattice& L, int prec, cudaStream_t st) {
+int launch_face_values(const Lattice& L, int prec, bool moments, cudaStream_t st) {
     if (L.per[2] || !L.P.open_extrap) return 0;
     if (L.P.open[0] != 1 && L.P.open[0] != 2 && L.P.open[1] != 1 && L.P.open[1] != 2) return 0;
     dim3 g((unsigned)((L.nx + 127) / 128), (unsigned)L.ny, 2);
-    DISPATCH(prec, (k_face_values<P><<<g, 128, 0, st>>>(L)));
+    if (moments) {
+        DISPATCH(prec, (k_face_values<P, true><<<g, 128, 0, st>>>(L)));
+    } else {
+        DISPATCH(prec, (k_face_values<P, false><<<g, 128, 0, st>>>(L)));
+    }
     return 1;
 }
 

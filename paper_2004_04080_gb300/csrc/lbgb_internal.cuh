@@ -259,6 +259,7 @@ struct Lattice {
     double inv_nu[2];  // 1/nu_k, nu_k = (tau_k - 1/2)/3
     int tau_equal;     // tau_A == tau_B
     ParamsF PF;        // FP32 copies (see ParamsF)
+    float rref[2];     // about the mean initial density: the moment kernel sums deviations from it
     int* ipos;         // [n][3] floor of the position (FP32 geometry origin)
     float* fsnap;      // [n][9] position - ipos, v(t-1/2), omega(t-1/2) in FP32
     double* red;       // reduction partials
@@ -580,6 +581,20 @@ __device__ __forceinline__ void acc_add(const Lattice& L, unsigned long long* a,
     if (acc_words(L, v, w)) acc_add_words(L, a, w);
 }
 
+// Add the link force and torque of one site (Eqs. 22, 23) to the fixed-point
+// sums of F_liq, T_liq of its particle (p < 0: no link of the site reaches a
+// particle).  Integer atomics: the sums do not depend on the order of the
+// additions, so they are the same bits on every run.
+template <typename C>
+__device__ __forceinline__ void commit_link_forces(const Lattice& L, int p, const C (&F)[3], const C (&T)[3]) {
+    if (p < 0) return;
+#pragma unroll
+    for (int d = 0; d < 3; d++) {
+        acc_add(L, acc_slot(L, ACC_FLIQ, p, d), F[d]);
+        acc_add(L, acc_slot(L, ACC_TLIQ, p, d), T[d]);
+    }
+}
+
 __device__ __forceinline__ double acc_value(const Lattice& L, const unsigned long long* a) {
     if (!L.acc_wide) return (double)(long long)a[0] * 9.094947017729282e-13;  // 2^-40
     return (double)(long long)a[0] * 5.9604644775390625e-08 + (double)a[1] * 5.421010862427522e-20;
@@ -666,10 +681,17 @@ inline int kernel_setup(int threads, size_t smem) {
 // kernel launchers (each returns the number of kernels it launched)
 int launch_init_fields(const Lattice& L, int prec, const double* stage, cudaStream_t st);
 int launch_fluid_step(const Lattice& L, int prec, cudaStream_t st);
+// one step at tau = 1 from the moments psi, mom of time t to psi_o, mom_o
+// of time t + 1 (lbgb_moment.cu)
+int launch_moments(const Lattice& L, void* psi_o, void* mom_o, cudaStream_t st);
 // the one-component fluid (lbgb_single.cu)
 int launch_single_init(const Lattice& L, int prec, const double* stage, cudaStream_t st);
 int launch_single_step(const Lattice& L, int prec, cudaStream_t st);
-int launch_single_face_values(const Lattice& L, int prec, cudaStream_t st);
+// with the moments of a run at tau = 1: rho and j from the populations, the
+// push of the populations from rho and j, the face values from rho
+int launch_single_moments(const Lattice& L, int prec, cudaStream_t st);
+int launch_single_push(const Lattice& L, int prec, cudaStream_t st);
+int launch_single_face_values(const Lattice& L, int prec, bool moments, cudaStream_t st);
 int launch_single_fields_out(const Lattice& L, int prec, double* stage, cudaStream_t st);
 int launch_single_totals_partial(const Lattice& L, int prec, cudaStream_t st);
 int launch_single_populations_out(const Lattice& L, int prec, int i, double* stage, cudaStream_t st);
@@ -679,7 +701,7 @@ int launch_wall_bounce(const Lattice& L, int prec, cudaStream_t st);
 int launch_shell_density(const Lattice& L, int prec, cudaStream_t st);
 int launch_density(const Lattice& L, int prec, cudaStream_t st);
 int launch_wall_psi(const Lattice& L, int prec, cudaStream_t st);
-int launch_face_values(const Lattice& L, int prec, cudaStream_t st);
+int launch_face_values(const Lattice& L, int prec, bool moments, cudaStream_t st);
 int launch_fields_out(const Lattice& L, int prec, double* stage, cudaStream_t st);
 int launch_totals(const Lattice& L, int prec, double* out_dev, cudaStream_t st);
 int launch_populations_out(const Lattice& L, int prec, int k, int i, double* stage, cudaStream_t st);
@@ -689,7 +711,8 @@ int launch_map_initial(const Lattice& L, int prec, int first, int count, cudaStr
 // the link classes nb: of every site (full), or around the nodes the remap
 // of this step listed
 int launch_link_classes(const Lattice& L, bool full, cudaStream_t st);
-int launch_remap(const Lattice& L, int prec, int maxc, cudaStream_t st);
+// (moments: the state is psi and mom of a run at tau = 1, not the populations)
+int launch_remap(const Lattice& L, int prec, int maxc, bool moments, cudaStream_t st);
 int launch_virtual(const Lattice& L, int prec, int store_terms, cudaStream_t st);
 // Eqs. 26-27 and the side walls into Fpair (reads positions and velocities only)
 int launch_pairs(const Lattice& L, void* cells, size_t cell_cap, bool force_build, cudaStream_t st);

@@ -49,22 +49,47 @@ __device__ __forceinline__ typename Prec<PREC>::C node_rho1(const Lattice& L, lo
 // boundary node b and the next interior node b + 1 along z (Sec. 2.2),
 // rho_w = rho_b + (rho_b - rho_{b+1}) / 2 (rho_b alone for nz < 2), one
 // thread per column of face blockIdx.z, into element 0 of the face record
-template <int PREC>
+// (MOM: from the densities of a run at tau = 1)
+template <int PREC, bool MOM>
 __global__ void k1_face_values(Lattice L) {
     typedef typename Prec<PREC>::C C;
     const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y, side = blockIdx.z;
     if (x >= L.nx || L.P.open[side] != 2) return;
     const long long nxy = (long long)L.nx * L.ny, col = (long long)x + (long long)L.nx * y;
     const int zb = side == 0 ? 0 : L.nz - 1, zi = side == 0 ? 1 : L.nz - 2;
-    C r = node_rho1<PREC>(L, col + nxy * zb);
-    if (zi >= 0 && zi < L.nz) r += C(0.5) * (r - node_rho1<PREC>(L, col + nxy * zi));
+    const C* rho = (const C*)L.psi;
+    C r = MOM ? rho[col + nxy * zb] : node_rho1<PREC>(L, col + nxy * zb);
+    if (zi >= 0 && zi < L.nz) r += C(0.5) * (r - (MOM ? rho[col + nxy * zi] : node_rho1<PREC>(L, col + nxy * zi)));
     ((C*)L.face)[5 * (side * nxy + col)] = r;
+}
+
+// rho and j (Eqs. 6, 7) of every site into psi [N] and mom [3][pstride]
+template <int PREC>
+__global__ void k1_density(Lattice L) {
+    typedef typename Prec<PREC>::S S;
+    typedef typename Prec<PREC>::C C;
+    const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= L.N) return;
+    const S* f = (const S*)L.f_cur;
+    C rho = 0, j[3] = {0, 0, 0};
+#pragma unroll
+    for (int i = 0; i < Q; i++) {
+        const C v = ld_pop(f + pop1_index(i, s, L.pstride), pop_shift<S, C>(L, 0, i));
+        rho += v;
+        if (cx(i)) j[0] += C(cx(i)) * v;
+        if (cy(i)) j[1] += C(cy(i)) * v;
+        if (cz(i)) j[2] += C(cz(i)) * v;
+    }
+    if (!(rho > C(0) && rho < C(1e30))) atomicOr(L.flags, FLAG_NONFINITE);
+    ((C*)L.psi)[s] = rho;
+#pragma unroll
+    for (int d = 0; d < 3; d++) ((C*)L.mom)[d * L.pstride + s] = j[d];
 }
 
 // One time step of every site (grid: x chunks, y, z).  UNIT: omega = 1, so
 // Eq. 16 is f* = f^eq(rho, u + g) and the populations enter only through
-// their moments.
-template <int PREC, bool UNIT, bool SR>
+// their moments; MOM (with UNIT): these are read from psi and mom.
+template <int PREC, bool UNIT, bool SR, bool MOM>
 __global__ void __launch_bounds__(128) k1_step(Lattice L) {
     typedef typename Prec<PREC>::S S;
     typedef typename Prec<PREC>::C C;
@@ -75,16 +100,22 @@ __global__ void __launch_bounds__(128) k1_step(Lattice L) {
     const long long ps = L.pstride;
     const S* fc = (const S*)L.f_cur;
     C f[Q];
-#pragma unroll
-    for (int i = 0; i < Q; i++) f[i] = ld_pop(fc + pop1_index(i, s, ps), pop_shift<S, C>(L, 0, i));
-    // Eqs. 6, 7
     C rho = 0, j[3] = {0, 0, 0};
+    if constexpr (MOM) {
+        rho = ((const C*)L.psi)[s];
 #pragma unroll
-    for (int i = 0; i < Q; i++) {
-        rho += f[i];
-        if (cx(i)) j[0] += C(cx(i)) * f[i];
-        if (cy(i)) j[1] += C(cy(i)) * f[i];
-        if (cz(i)) j[2] += C(cz(i)) * f[i];
+        for (int d = 0; d < 3; d++) j[d] = ((const C*)L.mom)[d * ps + s];
+    } else {
+#pragma unroll
+        for (int i = 0; i < Q; i++) f[i] = ld_pop(fc + pop1_index(i, s, ps), pop_shift<S, C>(L, 0, i));
+        // Eqs. 6, 7
+#pragma unroll
+        for (int i = 0; i < Q; i++) {
+            rho += f[i];
+            if (cx(i)) j[0] += C(cx(i)) * f[i];
+            if (cy(i)) j[1] += C(cy(i)) * f[i];
+            if (cz(i)) j[2] += C(cz(i)) * f[i];
+        }
     }
     if (!(rho > C(0) && rho < C(1e30))) atomicOr(L.flags, FLAG_NONFINITE);
     const C ir = C(1) / rho;
@@ -249,27 +280,40 @@ int launch_single_init(const Lattice& L, int prec, const double* stage, cudaStre
     return 1;
 }
 
-int launch_single_face_values(const Lattice& L, int prec, cudaStream_t st) {
+int launch_single_face_values(const Lattice& L, int prec, bool moments, cudaStream_t st) {
     if (L.per[2] || !L.P.open_extrap || (L.P.open[0] != 2 && L.P.open[1] != 2)) return 0;
     dim3 g((unsigned)((L.nx + 127) / 128), (unsigned)L.ny, 2);
-    DISPATCH1(prec, (k1_face_values<P><<<g, 128, 0, st>>>(L)));
+    if (moments) {
+        DISPATCH1(prec, (k1_face_values<P, true><<<g, 128, 0, st>>>(L)));
+    } else {
+        DISPATCH1(prec, (k1_face_values<P, false><<<g, 128, 0, st>>>(L)));
+    }
+    return 1;
+}
+
+int launch_single_moments(const Lattice& L, int prec, cudaStream_t st) {
+    DISPATCH1(prec, (k1_density<P><<<nblk1(L.N, 256), 256, 0, st>>>(L)));
+    return 1;
+}
+
+template <int P, bool SR, bool MOM>
+static int launch_single_step_t(const Lattice& L, cudaStream_t st) {
+    const int bx = L.nx >= 128 ? 128 : ((L.nx + 31) / 32) * 32;
+    const dim3 g((unsigned)((L.nx + bx - 1) / bx), (unsigned)L.ny, (unsigned)L.nz);
+    if (MOM || L.P.tau[0] == 1.0) k1_step<P, true, SR, MOM><<<g, bx, 0, st>>>(L);
+    else k1_step<P, false, SR, false><<<g, bx, 0, st>>>(L);
     return 1;
 }
 
 int launch_single_step(const Lattice& L, int prec, cudaStream_t st) {
-    const int bx = L.nx >= 128 ? 128 : ((L.nx + 31) / 32) * 32;
-    const dim3 g((unsigned)((L.nx + bx - 1) / bx), (unsigned)L.ny, (unsigned)L.nz);
-    const bool unit = L.P.tau[0] == 1.0;
-    if (prec == LB_FP16 && L.sr) {
-        if (unit) k1_step<LB_FP16, true, true><<<g, bx, 0, st>>>(L);
-        else k1_step<LB_FP16, false, true><<<g, bx, 0, st>>>(L);
-        return 1;
-    }
-    if (unit) {
-        DISPATCH1(prec, (k1_step<P, true, false><<<g, bx, 0, st>>>(L)));
-    } else {
-        DISPATCH1(prec, (k1_step<P, false, false><<<g, bx, 0, st>>>(L)));
-    }
+    if (prec == LB_FP16 && L.sr) return launch_single_step_t<LB_FP16, true, false>(L, st);
+    DISPATCH1(prec, (launch_single_step_t<P, false, false>(L, st)));
+    return 1;
+}
+
+int launch_single_push(const Lattice& L, int prec, cudaStream_t st) {
+    if (prec == LB_FP16 && L.sr) return launch_single_step_t<LB_FP16, true, true>(L, st);
+    DISPATCH1(prec, (launch_single_step_t<P, false, true>(L, st)));
     return 1;
 }
 
