@@ -669,48 +669,32 @@ __global__ void k_link_classes_changed(Lattice L) {
 }
 
 // ------------------------------------------------------------ wetting
-// Indices of the 18 neighbours of a site (-1 beyond a wall) and the bit set
-// of those that are particle nodes; the 18 mask loads are independent, so
-// they are in flight together.
-__device__ __forceinline__ uint32_t nbr_solid(const Lattice& L, const SiteNbr& n, int (&m)[Q]) {
-    uint32_t bits = 0;
-#pragma unroll
-    for (int i = 1; i < Q; i++) {
-        bool wall = nbr_is_wall(n, i);
-        m[i] = wall ? -1 : (int)nbr_index(L, n, i);
-        uint8_t v = wall ? 0 : __ldg(L.mask + m[i]);
-        bits |= (uint32_t)(v != 0) << i;
-    }
-    return bits;
-}
-
 // Eq. 20 on every frontier node s (a particle node with at least one fluid
 // neighbour): psi^k(s) = (1 + zeta^k) sum w_i rho^k / sum w_i over the fluid
 // neighbours (with the Janus switch s of the node: 1 + s zeta^A, 1 - s zeta^B)
 // neighbours, and Eq. 21 (repulsive sign):
 // F_s = -G sum_k psi^k(s) sum w_i rho^kbar(s + c_i) c_i, added with its torque
 // (x_s - r_p) x F_s to the fixed-point sums F_s, T_s of the owning particle
-// (the step zeroes them in launch_remap).  A block loads psi^k and the owner
-// map of a 32 x 8 tile (+ one-site ring) for all planes of its z chunk (+ one
-// on each side) into shared memory in one batch, 12 bytes per site in
-// coalesced rows; the frontier nodes of the chunk (from the link classes)
-// are then packed onto consecutive threads, so that the per-node work runs
-// with all lanes busy, and each takes its fluid neighbours from shared
-// memory.  The densities rho^k of the fluid nodes are those of the full
-// density pass of this step (k_density).
-constexpr int VTX = 32, VTY = 8, VZC = 8;  // tile and planes per block
+// (zero at the start of the step).  The link classes of a particle node are
+// the links to its fluid neighbours, so a block reads the link classes of a
+// 32 x 8 tile for a chunk of planes (4 bytes a site), packs the frontier nodes
+// onto consecutive threads, and each thread gathers the densities of its
+// node's fluid neighbours (a third of the 18), which are those of the fluid
+// nodes at this time.  It is bound by the latency of these gathers and by
+// issue (55 %).  (Copying psi and the owner map of the tile and its ring to
+// shared memory instead moved 20 bytes a site for the 6 % of the sites that
+// are frontier nodes: 512 x 512 x 256, 14,444 particles, 530 us against 298
+// now; 96^3 FP64 115 against 88, with sums in integer weights.)
+constexpr int VTX = 32, VTY = 8, VZC = 16;  // tile and planes per block (4096 sites: 12 bits of an entry)
 
 template <int PREC>
-__global__ void __launch_bounds__(VTX* VTY) k_virtual(Lattice L, int store_terms, int zc) {
+__global__ void __launch_bounds__(VTX* VTY) k_virtual(const __grid_constant__ Lattice L, int store_terms, int zc) {
     typedef typename Prec<PREC>::C C;
-    constexpr int NT = VTX * VTY, NPL = VZC + 2;
-    extern __shared__ __align__(16) unsigned char vsm[];
-    // planes z0-1 .. z0+zc of the tile + ring: node codes, then psi^A, psi^B
-    int (*snd)[VTY + 2][VTX + 2] = reinterpret_cast<int (*)[VTY + 2][VTX + 2]>(vsm);
-    // (psi^A, psi^B) pairs after the node codes (whose size is a multiple of 16 bytes)
-    C (*sp)[VTY + 2][VTX + 2][2] =
-        reinterpret_cast<C (*)[VTY + 2][VTX + 2][2]>(vsm + sizeof(int) * NPL * (VTY + 2) * (VTX + 2));
-    __shared__ int cand[NT * VZC];
+    struct alignas(2 * sizeof(C)) Pair {
+        C a, b;
+    };
+    constexpr int NT = VTX * VTY;
+    __shared__ unsigned cand[NT * VZC];  // link bits 1..18 above the site's place in the tile
     __shared__ int wcnt[NT / 32];
 
     const int x0 = blockIdx.x * VTX, y0 = blockIdx.y * VTY;
@@ -720,54 +704,17 @@ __global__ void __launch_bounds__(VTX* VTY) k_virtual(Lattice L, int store_terms
     const bool act = tx < W && ty < H;
     const long long nxy = (long long)L.nx * L.ny;
     C* psi = (C*)L.psi;
-    auto wrap_xy = [&](int lx, int ly) {
-        int X = x0 + lx, Y = y0 + ly;
-        X = X < 0 ? X + L.nx : (X >= L.nx ? X - L.nx : X);
-        Y = Y < 0 ? Y + L.ny : (Y >= L.ny ? Y - L.ny : Y);
-        return X + L.nx * Y;
-    };
-    const int own_xy = wrap_xy(tx, ty);
-    const bool has_ring = tid < 2 * (W + 2) + 2 * H;
-    int rlx, rly;
-    if (tid < W + 2) { rlx = tid - 1; rly = -1; }
-    else if (tid < 2 * (W + 2)) { rlx = tid - (W + 2) - 1; rly = H; }
-    else if (tid < 2 * (W + 2) + H) { rlx = -1; rly = tid - 2 * (W + 2); }
-    else { rlx = W; rly = tid - 2 * (W + 2) - H; }
-    const int ring_xy = has_ring ? wrap_xy(rlx, rly) : 0;
-    // every plane of the chunk at once (asynchronous copies, all in flight
-    // together); a plane beyond a wall has no fluid node
-    for (int q = 0; q < nz_b + 2; q++) {
-        const int p = z0 - 1 + q;
-        const bool wall = (p < 0 || p >= L.nz) && !L.per[2];
-        const int Z = p < 0 ? p + L.nz : (p >= L.nz ? p - L.nz : p);
-        const long long zoff = nxy * Z;
-        auto put = [&](int ly, int lx, long long g) {
-            if (wall) {
-                snd[q][ly][lx] = ND_WALL;
-                sp[q][ly][lx][0] = sp[q][ly][lx][1] = C(0);
-                return;
-            }
-            cp_async_4(&snd[q][ly][lx], L.owner + g);
-            if (sizeof(C) == 8) {
-                cp_async_16(&sp[q][ly][lx][0], psi + 2 * g);
-            } else {
-                cp_async_8(&sp[q][ly][lx][0], psi + 2 * g);
-            }
-        };
-        if (act) put(ty + 1, tx + 1, zoff + own_xy);
-        if (has_ring) put(rly + 1, rlx + 1, zoff + ring_xy);
-    }
+    const int own_xy = act ? x0 + tx + L.nx * (y0 + ty) : 0;
     // the frontier nodes of the tile's own column (a particle node with a
     // fluid neighbour: its link classes), one bit per plane of the chunk
     unsigned front = 0;
-    if (act)
-        for (int q = 1; q <= nz_b; q++) {
-            const uint32_t c = L.nb[nxy * (z0 + q - 1) + own_xy];
-            front |= (unsigned)((c & NB_SOLID) && (c & NB_LINKS)) << q;
-        }
-    cp_async_commit();
-    cp_async_wait_all();
-    __syncthreads();
+    uint32_t c[VZC];
+#pragma unroll
+    for (int q = 0; q < VZC; q++) c[q] = act && q < nz_b ? L.nb[nxy * (z0 + q) + own_xy] : 0u;
+    {
+#pragma unroll
+        for (int q = 0; q < VZC; q++) front |= (unsigned)((c[q] & NB_SOLID) && (c[q] & NB_LINKS)) << q;
+    }
     // the frontier nodes of the chunk, packed onto consecutive threads (in
     // plane, warp and lane order: fixed by the geometry)
     const int mine = __popc(front);
@@ -785,43 +732,52 @@ __global__ void __launch_bounds__(VTX* VTY) k_virtual(Lattice L, int store_terms
         off += w < warp ? wcnt[w] : 0;
         tot += wcnt[w];
     }
-    for (int q = 1; q <= nz_b; q++)
-        if ((front >> q) & 1u) cand[off++] = q * NT + tid;
+#pragma unroll
+    for (int q = 0; q < VZC; q++)
+        if ((front >> q) & 1u) cand[off++] = (c[q] & NB_LINKS) << 12 | (unsigned)(q * NT + tid);
     __syncthreads();
-    const C G = prm<C>(L.P.G, L.PF.G), zA = C(1) + C(L.P.zeta[0]), zB = C(1) + C(L.P.zeta[1]);
+    const C G36 = -prm<C>(L.P.G, L.PF.G) / C(36), zA = C(1) + C(L.P.zeta[0]), zB = C(1) + C(L.P.zeta[1]);
     // whole warps step through the list together (lanes past its end carry
-    // no term), so that a warp whose nodes all belong to one particle adds
-    // its terms with one set of atomics: the fixed-point words are summed
-    // across the warp first (exact integer sums, so the bits do not depend
-    // on the grouping)
+    // no term) for the sums over runs of lanes
     for (int base = warp * 32; base < tot; base += NT) {
         const int k = base + lane;
         bool has = false;
         int p = -1;
         C fs[3] = {0, 0, 0}, tq[3] = {0, 0, 0};
         if (k < tot) {
-            const int e = cand[k], q = e / NT, t = e - q * NT, cx0 = t % VTX, cy0 = t / VTX;
-            p = snd[q][cy0 + 1][cx0 + 1];
-            C num[2] = {0, 0}, den = 0;
+            const unsigned e = cand[k], fluid = e >> 12;
+            const int q = (int)(e & 4095u) / NT, t = (int)(e & 4095u) % NT, x = x0 + t % VTX, y = y0 + t / VTX, z = z0 + q;
+            const unsigned s = (unsigned)(x + L.nx * y) + (unsigned)nxy * (unsigned)z;
+            p = L.owner[s];
+            const int nxi = L.nx, pl = (int)nxy;
+            const int dxp = x == nxi - 1 ? 1 - nxi : 1, dxm = x == 0 ? nxi - 1 : -1;
+            const int dyp = y == L.ny - 1 ? nxi - pl : nxi, dym = y == 0 ? pl - nxi : -nxi;
+            const int dzp = z == L.nz - 1 ? pl - (int)L.N : pl, dzm = z == 0 ? (int)L.N - pl : -pl;
+            Pair r[Q];
+#pragma unroll
+            for (int i = 1; i < Q; i++) {
+                const int o = (cx(i) > 0 ? dxp : (cx(i) < 0 ? dxm : 0)) + (cy(i) > 0 ? dyp : (cy(i) < 0 ? dym : 0)) +
+                              (cz(i) > 0 ? dzp : (cz(i) < 0 ? dzm : 0));
+                r[i] = Pair{C(0), C(0)};
+                if ((fluid >> i) & 1u) r[i] = reinterpret_cast<const Pair*>(psi)[s + (unsigned)o];
+            }
+            // sums in units of 1/36 (weights 2 and 1)
+            C num[2] = {0, 0};
             C sA[3] = {0, 0, 0}, sB[3] = {0, 0, 0};
 #pragma unroll
             for (int i = 1; i < Q; i++) {
-                const int a = q + cz(i), yy = cy0 + 1 + cy(i), xx = cx0 + 1 + cx(i);
-                const bool fl = snd[a][yy][xx] == ND_FLUID;
-                C ra = fl ? sp[a][yy][xx][0] : C(0), rb = fl ? sp[a][yy][xx][1] : C(0);
-                C w = fl ? wgt<C>(i) : C(0);
-                num[0] += w * ra;
-                num[1] += w * rb;
-                den += w;
-                sA[0] += w * ra * C(cx(i)); sA[1] += w * ra * C(cy(i)); sA[2] += w * ra * C(cz(i));
-                sB[0] += w * rb * C(cx(i)); sB[1] += w * rb * C(cy(i)); sB[2] += w * rb * C(cz(i));
+                const C ra = i <= 6 ? C(2) * r[i].a : r[i].a, rb = i <= 6 ? C(2) * r[i].b : r[i].b;
+                num[0] += ra;
+                num[1] += rb;
+                if (cx(i)) sA[0] += C(cx(i)) * ra, sB[0] += C(cx(i)) * rb;
+                if (cy(i)) sA[1] += C(cy(i)) * ra, sB[1] += C(cy(i)) * rb;
+                if (cz(i)) sA[2] += C(cz(i)) * ra, sB[2] += C(cz(i)) * rb;
             }
+            const C den = C(2 * __popc(fluid & 0x7eu) + __popc(fluid & 0x7ff80u));
             if (den > C(0)) {
-                const int z = z0 + q - 1;
-                const long long s = nxy * z + (x0 + cx0) + (long long)L.nx * (y0 + cy0);
                 C d[3];
                 // x_s - r_p (minimum image) from the integer cell and offset of r_p
-                const int xs[3] = {x0 + cx0, y0 + cy0, z}, Ls[3] = {L.nx, L.ny, L.nz};
+                const int xs[3] = {x, y, z}, Ls[3] = {L.nx, L.ny, L.nz};
 #pragma unroll
                 for (int c = 0; c < 3; c++) {
                     int ip;
@@ -847,46 +803,20 @@ __global__ void __launch_bounds__(VTX* VTY) k_virtual(Lattice L, int store_terms
                     fa = C(1) + sw * C(L.P.zeta[0]);
                     fb = C(1) - sw * C(L.P.zeta[1]);
                 }
-                const C pa = fa * num[0] / den;
-                const C pb = fb * num[1] / den;
-                psi[2 * s] = pa;
-                psi[2 * s + 1] = pb;
+                const C iden = C(1) / den, pa = fa * (num[0] * iden);
+                const C pb = fb * (num[1] * iden);
+                reinterpret_cast<Pair*>(psi)[s] = Pair{pa, pb};
                 if (store_terms) {
 #pragma unroll
-                    for (int c = 0; c < 3; c++) fs[c] = -G * pa * sB[c] + -G * pb * sA[c];
+                    for (int c = 0; c < 3; c++) fs[c] = G36 * (pa * sB[c] + pb * sA[c]);
                     crs<C>(d, fs, tq);
                     has = true;
                 }
             }
         }
         if (!store_terms) continue;  // uniform across the block
-        const unsigned any = __ballot_sync(0xffffffffu, has);
-        if (!any) continue;
-        const int p0 = __shfl_sync(0xffffffffu, p, __ffs(any) - 1);
-        const bool one = __all_sync(0xffffffffu, !has || p == p0);
-#pragma unroll
-        for (int m = 0; m < 6; m++) {
-            const C v = m < 3 ? fs[m] : tq[m - 3];
-            unsigned long long w[2] = {0ull, 0ull};
-            if (has && !acc_words(L, v, w)) w[0] = w[1] = 0ull;
-            if (!one) {
-                if (has) acc_add_words(L, acc_slot(L, m < 3 ? ACC_FS : ACC_TS, p, m % 3), w);
-                continue;
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                w[0] += __shfl_xor_sync(0xffffffffu, w[0], o);
-                w[1] += __shfl_xor_sync(0xffffffffu, w[1], o);
-            }
-            if (lane == 0) acc_add_words(L, acc_slot(L, m < 3 ? ACC_FS : ACC_TS, p0, m % 3), w);
-        }
+        add_runs(L, ACC_FS, has ? p : -1, fs, tq);
     }
-}
-
-template <int PREC>
-size_t virtual_smem() {
-    typedef typename Prec<PREC>::C C;
-    return (size_t)(VZC + 2) * (VTY + 2) * (VTX + 2) * (sizeof(int) + 2 * sizeof(C));
 }
 
 // -------------------------------------------------------- pair forces
@@ -1256,10 +1186,13 @@ int launch_link_classes(const Lattice& L, bool full, cudaStream_t st) {
 
 int launch_virtual(const Lattice& L, int prec, int store_terms, cudaStream_t st) {
     if (L.nc <= 0) return 0;
-    const int zc = L.nz < VZC ? L.nz : VZC;
+    // full chunks where the lattice has blocks for all SMs several times over,
+    // thinner ones where it has not (32^3: 10.4 us with two chunks, 7.4 with 16)
+    const long long tiles = (long long)((L.nx + VTX - 1) / VTX) * ((L.ny + VTY - 1) / VTY);
+    const long long zw = tiles * L.nz / (4 * device_sms());
+    const int zc = (int)(zw < 2 ? 2 : (zw > VZC ? VZC : zw));
     dim3 grid((L.nx + VTX - 1) / VTX, (L.ny + VTY - 1) / VTY, (L.nz + zc - 1) / zc);
-    DISPATCHC(prec, (kernel_setup<k_virtual<P>>(VTX * VTY, virtual_smem<P>())));
-    DISPATCHC(prec, (k_virtual<P><<<grid, dim3(VTX, VTY), virtual_smem<P>(), st>>>(L, store_terms, zc)));
+    DISPATCHC(prec, (k_virtual<P><<<grid, dim3(VTX, VTY), 0, st>>>(L, store_terms, zc)));
     return 1;
 }
 

@@ -595,6 +595,38 @@ __device__ __forceinline__ void commit_link_forces(const Lattice& L, int p, cons
     }
 }
 
+// The forces F and torques T of the lanes of a whole warp (p: the lane's
+// particle, -1 none) added to the sums `term` and `term` + 1.  Lanes with one
+// particle mostly stand in runs: the words of a run are summed across its
+// lanes and added once (integer sums: the bits do not depend on the grouping).
+// exact: further forces in units of `unit`.
+template <typename C>
+__device__ __forceinline__ void add_runs(const Lattice& L, int term, int p, const C (&F)[3], const C (&T)[3],
+                                         const int* exact = nullptr, long long unit = 0) {
+    const int lane = threadIdx.x & 31;
+    const int before = __shfl_up_sync(0xffffffffu, p, 1), after = __shfl_down_sync(0xffffffffu, p, 1);
+    const unsigned heads = __ballot_sync(0xffffffffu, lane == 0 || before != p);
+    const int head = 31 - __clz(heads & (0xffffffffu >> (31 - lane)));
+    const bool tail = p >= 0 && (lane == 31 || after != p);
+    // the steps of the sum reach as far as the longest run
+    const int longest = __reduce_max_sync(0xffffffffu, lane - head);
+#pragma unroll
+    for (int m = 0; m < 6; m++) {
+        unsigned long long w[2] = {0ull, 0ull};
+        if (p >= 0 && !acc_words(L, m < 3 ? F[m] : T[m - 3], w)) w[0] = w[1] = 0ull;
+        if (m < 3 && exact) w[0] += (unsigned long long)(exact[m] * unit);
+        for (int o = 1; o <= longest; o <<= 1) {
+            const unsigned long long u = __shfl_up_sync(0xffffffffu, w[0], o);
+            if (lane - o >= head) w[0] += u;
+            if (sizeof(C) == 8) {
+                const unsigned long long v = __shfl_up_sync(0xffffffffu, w[1], o);
+                if (lane - o >= head) w[1] += v;
+            }
+        }
+        if (tail) acc_add_words(L, acc_slot(L, m < 3 ? term : term + 1, p, m % 3), w);
+    }
+}
+
 __device__ __forceinline__ double acc_value(const Lattice& L, const unsigned long long* a) {
     if (!L.acc_wide) return (double)(long long)a[0] * 9.094947017729282e-13;  // 2^-40
     return (double)(long long)a[0] * 5.9604644775390625e-08 + (double)a[1] * 5.421010862427522e-20;

@@ -824,24 +824,7 @@ __global__ void __launch_bounds__(128) k_bounce_links(const __grid_constant__ La
 #pragma unroll
             for (int d = 0; d < 3; d++) *mo = fmaf(j[d], h36, fmaf(j[d], l36, *mo)), mo += L.pstride;
         }
-        // runs of lanes with one particle: inclusive sums within the run, the
-        // last lane of a run adds them
-        const int before = __shfl_up_sync(0xffffffffu, p, 1), after = __shfl_down_sync(0xffffffffu, p, 1);
-        const unsigned heads = __ballot_sync(0xffffffffu, lane == 0 || before != p);
-        const int head = 31 - __clz(heads & (0xffffffffu >> (31 - lane)));
-        const bool tail = p >= 0 && (lane == 31 || after != p);
-#pragma unroll
-        for (int m = 0; m < 6; m++) {
-            unsigned long long w[2] = {0ull, 0ull};
-            if (p >= 0 && !acc_words(L, m < 3 ? F[m] : T[m - 3], w)) w[0] = 0ull;
-            if (m < 3) w[0] += (unsigned long long)(exact[m] * unit);
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const unsigned long long u = __shfl_up_sync(0xffffffffu, w[0], o);
-                if (lane - o >= head) w[0] += u;
-            }
-            if (tail) atomicAdd(acc_slot(L, m < 3 ? ACC_FLIQ : ACC_TLIQ, p, m % 3), w[0]);
-        }
+        add_runs(L, ACC_FLIQ, p, F, T, exact, unit);
     }
 }
 
