@@ -605,6 +605,7 @@ int lb_step(lb_ctx* ctx, int nsteps) {
         }
         ctx->stepped = 1;
     }
+    if (nsteps > 0) launch_clear_terms(L, s);
     for (int t = 0; L.ncomp == 2 && t < nsteps; t++) {
         int n = 0;
         const bool rec = ctx->rec_left > 0;

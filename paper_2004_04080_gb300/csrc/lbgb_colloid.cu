@@ -1029,97 +1029,99 @@ __global__ void __launch_bounds__(128) k_pairs(Lattice L) {
 }
 
 // --------------------------------------------------------- integrator
-// Eq. 33: qdot = 1/2 q (0, w*) written out component-wise
-__device__ __forceinline__ void qrate(const double (&q)[4], const double (&w)[3], double (&qd)[4]) {
-    qd[0] = 0.5 * (-q[1] * w[0] - q[2] * w[1] - q[3] * w[2]);
-    qd[1] = 0.5 * (q[0] * w[0] - q[3] * w[1] + q[2] * w[2]);
-    qd[2] = 0.5 * (q[3] * w[0] + q[0] * w[1] - q[1] * w[2]);
-    qd[3] = 0.5 * (-q[2] * w[0] + q[1] * w[1] + q[0] * w[2]);
-}
-
-// body-frame angular velocity R(q/|q|)^T w, R from Eq. 31
-__device__ __forceinline__ void to_body(const double (&q)[4], const double (&w)[3], double (&wb)[3]) {
-    double nq = sqrt(q[0] * q[0] + q[1] * q[1] + q[2] * q[2] + q[3] * q[3]);
-    double a = q[0] / nq, b = q[1] / nq, c = q[2] / nq, e = q[3] / nq;
-    double R00 = a * a + b * b - c * c - e * e, R01 = 2.0 * (b * c - a * e), R02 = 2.0 * (b * e + a * c);
-    double R10 = 2.0 * (b * c + a * e), R11 = a * a - b * b + c * c - e * e, R12 = 2.0 * (c * e - a * b);
-    double R20 = 2.0 * (b * e - a * c), R21 = 2.0 * (c * e + a * b), R22 = a * a - b * b - c * c + e * e;
-    wb[0] = R00 * w[0] + R10 * w[1] + R20 * w[2];
-    wb[1] = R01 * w[0] + R11 * w[1] + R21 * w[2];
-    wb[2] = R02 * w[0] + R12 * w[1] + R22 * w[2];
-}
-
-// Eq. 35 totals, Eq. 32 leap-frog, Eq. 34 implicit mid-step quaternion
-// (iterated until the rate changes by <= 1e-14, at most 20 times); then the
-// FP32 snapshot of the new state.  A particle faster than 1/2 lattice unit
-// per step is reported (the remap assumes smaller moves).
-__global__ void k_integrate(Lattice L) {
-    int p = blockIdx.x * blockDim.x + threadIdx.x;
+// Eq. 35 totals, Eq. 32 leap-frog, Eqs. 33-34 quaternions; then the FP32
+// snapshot of the new state.  A particle faster than 1/2 lattice unit per step
+// is reported (the remap assumes smaller moves).  The step's fixed-point sums
+// are read and cleared for the next step, and the list of changed nodes
+// emptied.
+//
+// Eq. 33 is qdot = q (0, w*) / 2 with the body-frame w* = R(q/|q|)^T w, which
+// is (0, w) q / 2 with w in the space frame, linear in q, so the implicit
+// mid-step equation of Eq. 34, qdot = (0, w) (q + qdot / 2) / 2, has the closed
+// form qdot = ((0, w) q / 2 - w.w q / 8) / (1 + w.w / 16), the fixed point of
+// the iteration that Eq. 34 prescribes.  (Iterated, with two roots and eight
+// divisions in FP64 each time: 40 us a step whatever the number of particles,
+// FP64 running two lanes a cycle on an SM; 11 us now, in blocks of one warp.)
+__global__ void __launch_bounds__(32) k_integrate(const __grid_constant__ Lattice L) {
+    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p == 0) *L.nb_chg = 0;
     if (p >= L.nc) return;
-    double F[3], T[3];
-    bool first = !L.prev_valid[p];
-    // the step's fixed-point sums as FP64 terms
-    double* terms[ACC_TERMS] = {L.Fliq, L.Tliq, L.Fd, L.Td, L.Fc, L.Tc, L.Fs, L.Ts};
-    for (int t = 0; t < ACC_TERMS; t++)
-        for (int d = 0; d < 3; d++) terms[t][3 * p + d] = acc_value(L, acc_slot(L, t, p, d));
-    for (int d = 0; d < 3; d++) {
-        double fp = first ? L.Fliq[3 * p + d] : L.Fliq_prev[3 * p + d];
-        double tp = first ? L.Tliq[3 * p + d] : L.Tliq_prev[3 * p + d];
-        F[d] = 0.5 * (fp + L.Fliq[3 * p + d]) + L.Fd[3 * p + d] + L.Fc[3 * p + d] + L.Fs[3 * p + d] +
-               L.Fpair[3 * p + d];
-        T[d] = 0.5 * (tp + L.Tliq[3 * p + d]) + L.Td[3 * p + d] + L.Tc[3 * p + d] + L.Ts[3 * p + d];
-        L.Ftot[3 * p + d] = F[d];
-        L.Ttot[3 * p + d] = T[d];
-        L.Fliq_prev[3 * p + d] = L.Fliq[3 * p + d];
-        L.Tliq_prev[3 * p + d] = L.Tliq[3 * p + d];
-    }
-    L.prev_valid[p] = 1;
-    double m = L.mass[p];
-    int Ls[3] = {L.nx, L.ny, L.nz};
-    for (int d = 0; d < 3; d++) {
-        double v = L.vel[3 * p + d] + F[d] / m;
-        double r = L.pos[3 * p + d] + v;
-        if (L.per[d]) r = r - double(Ls[d]) * floor(r / double(Ls[d]));
-        L.vel[3 * p + d] = v;
-        L.pos[3 * p + d] = r;
-        if (!(fabs(v) < 0.5)) atomicOr(L.flags, FLAG_NONFINITE);
-    }
-    if (L.P.rotate) {
-        double R = L.rad[p];
-        double I = 0.4 * m * R * R;
-        double w[3], q[4], wb[3], qd[4], qh[4];
-        for (int d = 0; d < 3; d++) w[d] = L.omg[3 * p + d] + T[d] / I;
-        for (int d = 0; d < 4; d++) q[d] = L.quat[4 * p + d];
-        to_body(q, w, wb);
-        qrate(q, wb, qd);
-        for (int d = 0; d < 4; d++) qh[d] = q[d] + 0.5 * qd[d];
-        for (int it = 0; it < 20; it++) {
-            double nd[4], delta = 0.0;
-            to_body(qh, w, wb);
-            qrate(qh, wb, nd);
-            for (int d = 0; d < 4; d++) {
-                delta = fmax(delta, fabs(nd[d] - qd[d]));
-                qh[d] = q[d] + 0.5 * nd[d];
-                qd[d] = nd[d];
-            }
-            if (delta <= 1e-14) break;
+    double t[ACC_TERMS][3], Fp[3], Tp[3], pair[3], r[3], v[3], w[3], q[4];
+#pragma unroll
+    for (int a = 0; a < ACC_TERMS; a++)
+#pragma unroll
+        for (int d = 0; d < 3; d++) {
+            unsigned long long* slot = acc_slot(L, a, p, d);
+            t[a][d] = acc_value(L, slot);
+            slot[0] = slot[1] = 0ull;
         }
-        double nq = 0.0;
+    const bool first = !L.prev_valid[p];
+#pragma unroll
+    for (int d = 0; d < 3; d++) {
+        Fp[d] = L.Fliq_prev[3 * p + d];
+        Tp[d] = L.Tliq_prev[3 * p + d];
+        pair[d] = L.Fpair[3 * p + d];
+        r[d] = L.pos[3 * p + d];
+        v[d] = L.vel[3 * p + d];
+        w[d] = L.omg[3 * p + d];
+    }
+#pragma unroll
+    for (int d = 0; d < 4; d++) q[d] = L.quat[4 * p + d];
+    const double im = 1.0 / L.mass[p], R = L.rad[p];
+    double* terms[ACC_TERMS] = {L.Fliq, L.Tliq, L.Fd, L.Td, L.Fc, L.Tc, L.Fs, L.Ts};
+#pragma unroll
+    for (int a = 0; a < ACC_TERMS; a++)
+#pragma unroll
+        for (int d = 0; d < 3; d++) terms[a][3 * p + d] = t[a][d];
+    const int Ls[3] = {L.nx, L.ny, L.nz};
+    bool fast = false;
+    double T[3];
+#pragma unroll
+    for (int d = 0; d < 3; d++) {
+        const double fp = first ? t[ACC_FLIQ][d] : Fp[d], tp = first ? t[ACC_TLIQ][d] : Tp[d];
+        const double F = 0.5 * (fp + t[ACC_FLIQ][d]) + t[ACC_FD][d] + t[ACC_FC][d] + t[ACC_FS][d] + pair[d];
+        T[d] = 0.5 * (tp + t[ACC_TLIQ][d]) + t[ACC_TD][d] + t[ACC_TC][d] + t[ACC_TS][d];
+        L.Ftot[3 * p + d] = F;
+        L.Ttot[3 * p + d] = T[d];
+        L.Fliq_prev[3 * p + d] = t[ACC_FLIQ][d];
+        L.Tliq_prev[3 * p + d] = t[ACC_TLIQ][d];
+        v[d] += F * im;
+        r[d] += v[d];
+        if (L.per[d] && !(r[d] >= 0.0 && r[d] < (double)Ls[d])) r[d] = r[d] - double(Ls[d]) * floor(r[d] / double(Ls[d]));
+        fast |= !(fabs(v[d]) < 0.5);
+        L.vel[3 * p + d] = v[d];
+        L.pos[3 * p + d] = r[d];
+    }
+    if (fast) atomicOr(L.flags, FLAG_NONFINITE);
+    L.prev_valid[p] = 1;
+    if (L.P.rotate) {
+        const double iI = im / (0.4 * R * R);
+        double ww = 0.0, nq = 0.0;
+#pragma unroll
+        for (int d = 0; d < 3; d++) {
+            w[d] += T[d] * iI;
+            ww += w[d] * w[d];
+            L.omg[3 * p + d] = w[d];
+        }
+        const double s = 1.0 / (1.0 + 0.0625 * ww);
+        const double wq[4] = {-(w[0] * q[1] + w[1] * q[2] + w[2] * q[3]), w[0] * q[0] + w[1] * q[3] - w[2] * q[2],
+                              w[1] * q[0] + w[2] * q[1] - w[0] * q[3], w[2] * q[0] + w[0] * q[2] - w[1] * q[1]};
+#pragma unroll
         for (int d = 0; d < 4; d++) {
-            q[d] = q[d] + qd[d];
+            q[d] += (0.5 * wq[d] - 0.125 * ww * q[d]) * s;
             nq += q[d] * q[d];
         }
-        nq = sqrt(nq);
-        for (int d = 0; d < 3; d++) L.omg[3 * p + d] = w[d];
-        for (int d = 0; d < 4; d++) L.quat[4 * p + d] = q[d] / nq;
+        const double in = 1.0 / sqrt(nq);
+#pragma unroll
+        for (int d = 0; d < 4; d++) L.quat[4 * p + d] = q[d] * in;
     }
+#pragma unroll
     for (int d = 0; d < 3; d++) {
-        double r = L.pos[3 * p + d];
-        int ip = (int)floor(r);
+        const int ip = (int)floor(r[d]);
         L.ipos[3 * p + d] = ip;
-        L.fsnap[9 * p + d] = float(r - (double)ip);
-        L.fsnap[9 * p + 3 + d] = float(L.vel[3 * p + d]);
-        L.fsnap[9 * p + 6 + d] = float(L.omg[3 * p + d]);
+        L.fsnap[9 * p + d] = float(r[d] - (double)ip);
+        L.fsnap[9 * p + 3 + d] = float(v[d]);
+        L.fsnap[9 * p + 6 + d] = float(w[d]);
     }
 }
 
@@ -1158,14 +1160,16 @@ static void launch_remap_t(const Lattice& L, cudaStream_t st) {
     k_remap_commit<P, MOM><<<grid, PBLK, 0, st>>>(L);
 }
 
-int launch_remap(const Lattice& L, int prec, int maxc, bool moments, cudaStream_t st) {
+int launch_clear_terms(const Lattice& L, cudaStream_t st) {
     if (L.nc <= 0) return 0;
-    // the per-particle terms of the step are fixed-point sums of block
-    // partials and per-site contributions (acc_add), from zero; the
-    // integrator turns them into F_liq, T_liq, F_d, T_d, F_c, T_c, F_s, T_s
-    (void)maxc;
     cudaMemsetAsync(L.acc, 0, (size_t)ACC_TERMS * L.maxc * 6 * sizeof(unsigned long long), st);
     cudaMemsetAsync(L.nb_chg, 0, sizeof(int), st);
+    return 0;
+}
+
+int launch_remap(const Lattice& L, int prec, int maxc, bool moments, cudaStream_t st) {
+    if (L.nc <= 0) return 0;
+    (void)maxc;
     if (moments) {
         DISPATCHC(prec, (launch_remap_t<P, true>(L, st)));
     } else {
@@ -1242,7 +1246,7 @@ int launch_pairs(const Lattice& L, void* cells, size_t cell_cap, bool force_buil
 
 int launch_integrate(const Lattice& L, cudaStream_t st) {
     if (L.nc <= 0) return 0;
-    k_integrate<<<(L.nc + 127) / 128, 128, 0, st>>>(L);
+    k_integrate<<<(L.nc + 31) / 32, 32, 0, st>>>(L);
     return 1;
 }
 

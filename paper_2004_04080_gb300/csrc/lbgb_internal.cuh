@@ -745,6 +745,9 @@ int launch_map_initial(const Lattice& L, int prec, int first, int count, cudaStr
 int launch_link_classes(const Lattice& L, bool full, cudaStream_t st);
 // (moments: the state is psi and mom of a run at tau = 1, not the populations)
 int launch_remap(const Lattice& L, int prec, int maxc, bool moments, cudaStream_t st);
+// the per-particle sums and the list of changed nodes, empty for the first step of a call
+// (k_integrate leaves them so for the next)
+int launch_clear_terms(const Lattice& L, cudaStream_t st);
 int launch_virtual(const Lattice& L, int prec, int store_terms, cudaStream_t st);
 // Eqs. 26-27 and the side walls into Fpair (reads positions and velocities only)
 int launch_pairs(const Lattice& L, void* cells, size_t cell_cap, bool force_build, cudaStream_t st);
