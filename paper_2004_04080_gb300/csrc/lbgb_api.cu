@@ -636,7 +636,7 @@ int lb_step(lb_ctx* ctx, int nsteps) {
             V.psi = run.psi[0];
             V.mom = run.mom[0];
         }
-        n += launch_remap(V, ctx->prec, ctx->maxc, kept, s);  // destroy / create (Eqs. 24, 25)
+        n += launch_remap(V, ctx->prec, kept, t == 0, s);  // destroy / create (Eqs. 24, 25)
         if (L.nc > 0) {
             n += launch_link_classes(V, !ctx->nb_valid, s);
             ctx->nb_valid = 1;

@@ -632,18 +632,6 @@ __device__ __forceinline__ double acc_value(const Lattice& L, const unsigned lon
     return (double)(long long)a[0] * 5.9604644775390625e-08 + (double)a[1] * 5.421010862427522e-20;
 }
 
-// Neumaier sum in the compute type (per-thread partials before the FP64 merge)
-template <typename C>
-struct CSum {
-    C s, c;
-    __device__ __forceinline__ void add(C x) {
-        C t = s + x;
-        if (fabs(s) >= fabs(x)) c += (s - t) + x;
-        else c += (x - t) + s;
-        s = t;
-    }
-};
-
 // asynchronous global -> shared copies (cp.async) and their completion
 __device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void cp_async_16(void* dst, const void* src) {
@@ -744,7 +732,8 @@ int launch_map_initial(const Lattice& L, int prec, int first, int count, cudaStr
 // of this step listed
 int launch_link_classes(const Lattice& L, bool full, cudaStream_t st);
 // (moments: the state is psi and mom of a run at tau = 1, not the populations)
-int launch_remap(const Lattice& L, int prec, int maxc, bool moments, cudaStream_t st);
+// wide: the first step of a call
+int launch_remap(const Lattice& L, int prec, bool moments, bool wide, cudaStream_t st);
 // the per-particle sums and the list of changed nodes, empty for the first step of a call
 // (k_integrate leaves them so for the next)
 int launch_clear_terms(const Lattice& L, cudaStream_t st);

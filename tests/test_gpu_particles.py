@@ -3,7 +3,7 @@ import numpy as np
 import pytest
 
 from paper_2004_04080_gb300.workloads import mixture_densities
-from test_gpu_parity import run_both
+from test_gpu_parity import compare_fields, run_both
 
 pytestmark = pytest.mark.gpu
 
@@ -28,3 +28,42 @@ def test_orientation_closed_form(spin, n):
     gc, rc = g.get_colloids(), o.get_colloids()
     assert np.abs(gc["quat"] - rc["quat"]).max() < 1e-13
     assert np.abs(np.linalg.norm(gc["quat"], axis=1) - 1.0).max() < 1e-15
+
+
+@pytest.mark.parametrize("prec,tol", [("fp64", 1e-12), ("fp32", 1e-5)])
+@pytest.mark.parametrize("calls", [(8,), (1,) * 8])
+@pytest.mark.parametrize("speed", [0.0, 0.02, 0.45])
+def test_remap_shell(speed, calls, prec, tol):
+    """Only nodes within |v| of a surface are looked at after the first step of
+    a call: slow and nearly fastest particles, across the periodic edges and
+    next to a wall, in one call and in calls of one step.  Bounds of the forms;
+    the node maps are equal."""
+    shape = (28, 19, 23)
+    vel = speed * np.array([[1.0, 0.0, 0.0], [-0.6, 0.0, 0.8], [0.0, -0.8, 0.6], [0.577, 0.577, -0.577]])
+    col = dict(pos=[[26.9, 3.2, 4.6], [8.3, 4.1, 6.2], [7.7, 14.2, 17.3], [20.4, 12.9, 15.1]],
+               radius=[3.1, 2.5, 3.4, 2.9], mass=[1e6] * 4, vel=vel, omega=[[0.0, 0.02, 0.01]] * 4)
+    params = dict(G=0.3, zeta=(0.05, -0.05), bc=(1, 1, 0))
+    dens = mixture_densities(shape, seed=5, amp=0.02)
+    g, o = run_both(shape, params, calls[0], prec, col, dens)
+    for n in calls[1:]:
+        g.step(n)
+        o.step(n)
+    compare_fields(g, o, tol)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_overlap_is_reported_by_every_call(prec):
+    """Particles that have run into each other are reported by the call in
+    which they meet and by the ones after it."""
+    from paper_2004_04080_gb300.lbgb import LBError, LBLattice
+
+    g = LBLattice((24, 16, 16), prec, max_colloids=2)
+    g.set_params(G=0.0)
+    g.init_fields(*mixture_densities((24, 16, 16), seed=5, amp=0.0))
+    g.add_colloids(pos=[[7.5, 8.1, 8.2], [14.9, 8.1, 8.2]], radius=[3.5, 3.5], mass=[1e6, 1e6],
+                   vel=[[0.1, 0.0, 0.0], [0.0, 0.0, 0.0]])
+    with pytest.raises(LBError):
+        g.step(12)
+    for _ in range(2):
+        with pytest.raises(LBError):
+            g.step(1)
