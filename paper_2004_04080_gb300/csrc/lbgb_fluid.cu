@@ -56,26 +56,30 @@ __global__ void k_density(Lattice L) {
         return;
     }
     const S* f = (const S*)L.f_cur;
-    C rho[2] = {0, 0}, jt[2][3] = {{0, 0, 0}, {0, 0, 0}};
+    // j from the differences of opposite links of both components (39
+    // additions; 60 link by link: 96^3 in FP64, which the additions bound, 182
+    // -> 147 us for the whole pass)
+    C rho[2] = {0, 0}, jt[3] = {0, 0, 0}, last[2] = {0, 0};
 #pragma unroll
     for (int i = 0; i < Q; i++) {
         C v[2];
         ld_pair(f + pair_index(i, s, L.pstride), pop_shift<S, C>(L, 0, i), pop_shift<S, C>(L, 1, i), v[0], v[1]);
 #pragma unroll
-        for (int k = 0; k < 2; k++) {
-            rho[k] += v[k];
-            if (MOM) {
-                if (cx(i) > 0) jt[k][0] += v[k]; else if (cx(i) < 0) jt[k][0] -= v[k];
-                if (cy(i) > 0) jt[k][1] += v[k]; else if (cy(i) < 0) jt[k][1] -= v[k];
-                if (cz(i) > 0) jt[k][2] += v[k]; else if (cz(i) < 0) jt[k][2] -= v[k];
-            }
+        for (int k = 0; k < 2; k++) rho[k] += v[k];
+        if (MOM && i > 0 && i == opp(i - 1)) {
+            const C d = (last[0] - v[0]) + (last[1] - v[1]);  // along c_(i - 1)
+            if (cx(i) < 0) jt[0] += d; else if (cx(i) > 0) jt[0] -= d;
+            if (cy(i) < 0) jt[1] += d; else if (cy(i) > 0) jt[1] -= d;
+            if (cz(i) < 0) jt[2] += d; else if (cz(i) > 0) jt[2] -= d;
         }
+        last[0] = v[0];
+        last[1] = v[1];
     }
     psi[2 * s] = rho[0];
     psi[2 * s + 1] = rho[1];
     if (MOM)
 #pragma unroll
-        for (int d = 0; d < 3; d++) mom[d * L.pstride + s] = jt[0][d] + jt[1][d];
+        for (int d = 0; d < 3; d++) mom[d * L.pstride + s] = jt[d];
     if (!(rho[0] >= C(0) && rho[1] >= C(0) && rho[0] < C(1e30) && rho[1] < C(1e30)))
         atomicOr(L.flags, FLAG_NONFINITE);
 }
@@ -406,26 +410,11 @@ __device__ __forceinline__ void collide_site(const Lattice& L, SH& sh, const int
     const unsigned bb = li.bb, pm = li.pm;
     const int p0 = li.p0;
     const bool multi = li.multi;
-    // Eq. 11 (repulsive sign) + body force from the shared-memory psi planes
-    C sA[3] = {0, 0, 0}, sB[3] = {0, 0, 0};
-#pragma unroll
-    for (int i = 1; i < Q; i++) {
-        int slot = sl[cz(i) + 1];
-        C pa = sh.psi[slot][0][ty + 1 + cy(i)][tx + 1 + cx(i)];
-        C pb = sh.psi[slot][1][ty + 1 + cy(i)][tx + 1 + cx(i)];
-        C w = wgt<C>(i);
-        if (cx(i)) { sA[0] += C(cx(i)) * w * pa; sB[0] += C(cx(i)) * w * pb; }
-        if (cy(i)) { sA[1] += C(cy(i)) * w * pa; sB[1] += C(cy(i)) * w * pb; }
-        if (cz(i)) { sA[2] += C(cz(i)) * w * pa; sB[2] += C(cz(i)) * w * pb; }
-    }
-    C F[2][3];
-    C G = prm<C>(L.P.G, L.PF.G);
-#pragma unroll
-    for (int d = 0; d < 3; d++) {
-        C g = prm<C>(L.P.body_force[d], L.PF.body_force[d]);
-        F[0][d] = -G * m.rho[0] * sB[d] + m.rho[0] * g;
-        F[1][d] = -G * m.rho[1] * sA[d] + m.rho[1] * g;
-    }
+    // Eq. 11 (repulsive sign) + body force from the shared-memory psi planes,
+    // per density: F^k / rho^k = g - G S
+    C grad[2][3];
+    link_gradient<C>(grad, [&](int i, int k) { return sh.psi[sl[cz(i) + 1]][k][ty + 1 + cy(i)][tx + 1 + cx(i)]; });
+    const C G36 = prm<C>(L.P.G, L.PF.G) * wgt<C>(7);
     if (!solid && !(m.rho[0] >= C(0) && m.rho[1] >= C(0) && m.rho[0] < C(1e30) && m.rho[1] < C(1e30)))
         atomicOr(L.flags, FLAG_NONFINITE);
     C u[3], om;
@@ -433,22 +422,31 @@ __device__ __forceinline__ void collide_site(const Lattice& L, SH& sh, const int
     C us[2][3];
     C tiny = sizeof(C) == 8 ? C(1e-300) : C(1e-30);
 #pragma unroll
-    for (int k = 0; k < 2; k++) {
-        C ir = m.rho[k] > tiny ? C(1) / m.rho[k] : C(0);
+    for (int k = 0; k < 2; k++)
 #pragma unroll
-        for (int d = 0; d < 3; d++) us[k][d] = u[d] + F[k][d] * ir;
-    }
+        for (int d = 0; d < 3; d++)
+            us[k][d] = u[d] + (m.rho[k] > tiny ? prm<C>(L.P.body_force[d], L.PF.body_force[d]) - G36 * grad[1 - k][d] : C(0));
     C uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
     C uus[2] = {us[0][0] * us[0][0] + us[0][1] * us[0][1] + us[0][2] * us[0][2],
                 us[1][0] * us[1][0] + us[1][1] * us[1][1] + us[1][2] * us[1][2]};
     C one_m_om = C(1) - om;
-    // 3 w_c rho^k per weight class c (1 axis, 2 diagonal): the wall term of
-    // the bounce-back (Eqs. 9, 17) is 3 w_c rho^k (-2 c_i.u_w)
-    C B[2][3];
+    // Eq. 5 per weight class c (1 axis, 2 diagonal) and opposite pair of links:
+    // f^eq(+-c_i, v) = w_c rho (1 - 3/2 v.v) + H_c (c_i.v)^2 +- B_c c_i.v with
+    // B_c = 3 w_c rho, H_c = 9/2 w_c rho.  The wall term of the bounce-back
+    // (Eqs. 9, 17) is B_c (-2 c_i.u_w).  Each product once for both links and
+    // none by a zero of c_i: the collision link by link took 2.3 times the
+    // operations (140 x 92 x 110, unequal tau, FP32: 140 -> 131 us a step).
+    C B[2][3], H[2][3], Ae[2][3], As[2][3];
 #pragma unroll
     for (int k = 0; k < 2; k++)
 #pragma unroll
-        for (int c = 0; c < 3; c++) B[k][c] = C(3) * (wgt<C>(c == 0 ? 0 : (c == 1 ? 1 : 7)) * m.rho[k]);
+        for (int c = 0; c < 3; c++) {
+            const C wr = wgt<C>(c == 0 ? 0 : (c == 1 ? 1 : 7)) * m.rho[k];
+            B[k][c] = C(3) * wr;
+            H[k][c] = C(4.5) * wr;
+            Ae[k][c] = wr * (C(1) - C(1.5) * uu);
+            As[k][c] = wr * (C(1) - C(1.5) * uus[k]);
+        }
     // site-index steps to the neighbours, periodic wrap folded in (32-bit:
     // a lattice holds fewer than 2^31 sites)
     const unsigned ps = (unsigned)L.pstride;
@@ -488,47 +486,57 @@ __device__ __forceinline__ void collide_site(const Lattice& L, SH& sh, const int
             st_pair(p, va, vb, sa, sb);
         }
     };
-#pragma unroll
-    for (int i = 0; i < Q; i++) {
-        C fs[2];
+    {
+        C f0[2];
 #pragma unroll
         for (int k = 0; k < 2; k++) {
-            fs[k] = one_m_om * (ld_pop(pop(k * Q + i), pop_shift<S, C>(L, k, i)) -
-                                feq<C>(i, m.rho[k], u[0], u[1], u[2], uu)) +
-                    feq<C>(i, m.rho[k], us[k][0], us[k][1], us[k][2], uus[k]);
+            f0[k] = one_m_om * (ld_pop(pop(k * Q), pop_shift<S, C>(L, k, 0)) - Ae[k][0]) + As[k][0];
+            if (solid) f0[k] = wgt<C>(0) * prm<C>(L.P.rho0[k], L.PF.rho0[k]);
         }
-        if (i == 0) {
-            put2(pair_at(0, (unsigned)SKEW + s), solid ? wgt<C>(0) * prm<C>(L.P.rho0[0], L.PF.rho0[0]) : fs[0],
-                 solid ? wgt<C>(0) * prm<C>(L.P.rho0[1], L.PF.rho0[1]) : fs[1], pop_shift<S, C>(L, 0, 0),
-                 pop_shift<S, C>(L, 1, 0));
-            continue;
-        }
-        const int lo = (i & 1) ? i : i - 1;  // first plane of the pair
-        const bool b = (bb >> i) & 1u;
-        const unsigned q = solid ? s
-                                 : s + (unsigned)((cx(i) > 0 ? dxp : (cx(i) < 0 ? dxm : 0)) +
-                                                  (cy(i) > 0 ? dyp : (cy(i) < 0 ? dym : 0)) +
-                                                  (cz(i) > 0 ? dzp : (cz(i) < 0 ? dzm : 0)));
-        // push: the destination's element of plane i, SKEW + q - c_ix (at the
-        // source's x); bounce-back: the own element of plane opp(i),
-        // SKEW + s + c_ix
-        const unsigned off = b ? (unsigned)(SKEW + cx(i)) + s + (opp(i) == lo ? 0u : ps)
-                               : (unsigned)(SKEW - cx(i)) + q + (i == lo ? 0u : ps);
-        const int zs = cz(i) + 1;
-        C cw = C(cx(i)) * V[zs][0] + C(cy(i)) * V[zs][1] + C(cz(i)) * V[zs][2];
-        cw = b ? C(-2) * cw : C(0);  // f_ibar = f*_i - 6 w_i rho c_i.u_w (Eq. 17)
-        const int c = i <= 6 ? 1 : 2;
-        C fb[2];
+        put2(pair_at(0, (unsigned)SKEW + s), f0[0], f0[1], pop_shift<S, C>(L, 0, 0), pop_shift<S, C>(L, 1, 0));
+    }
 #pragma unroll
-        for (int k = 0; k < 2; k++) fb[k] = fs[k] + B[k][c] * cw;
-        put2(pair_at(lo, off), solid ? wgt<C>(i) * prm<C>(L.P.rho0[0], L.PF.rho0[0]) : fb[0],
-             solid ? wgt<C>(i) * prm<C>(L.P.rho0[1], L.PF.rho0[1]) : fb[1], pop_shift<S, C>(L, 0, i),
-             pop_shift<S, C>(L, 1, i));
-        C fl = fs[0] + fb[0] + fs[1] + fb[1];
-        fl = (pm >> i) & 1u ? fl : C(0);
-        if (cx(i)) Fl[0] += C(cx(i)) * fl;
-        if (cy(i)) Fl[1] += C(cy(i)) * fl;
-        if (cz(i)) Fl[2] += C(cz(i)) * fl;
+    for (int lo = 1; lo < Q; lo += 2) {  // planes lo and opp(lo) = lo + 1
+        const int c = lo <= 6 ? 1 : 2;
+        const C cu = along<C>(lo, u);
+        C fp[2][2];
+#pragma unroll
+        for (int k = 0; k < 2; k++) {
+            const C cs = along<C>(lo, us[k]);
+            const C ee = Ae[k][c] + (H[k][c] * cu) * cu, es = As[k][c] + (H[k][c] * cs) * cs;
+            fp[0][k] = one_m_om * (ld_pop(pop(k * Q + lo), pop_shift<S, C>(L, k, lo)) - (ee + B[k][c] * cu)) +
+                       (es + B[k][c] * cs);
+            fp[1][k] = one_m_om * (ld_pop(pop(k * Q + lo + 1), pop_shift<S, C>(L, k, lo + 1)) - (ee - B[k][c] * cu)) +
+                       (es - B[k][c] * cs);
+        }
+#pragma unroll
+        for (int side = 0; side < 2; side++) {
+            const int i = lo + side;
+            const C(&fs)[2] = fp[side];
+            const bool b = (bb >> i) & 1u;
+            const unsigned q = solid ? s
+                                     : s + (unsigned)((cx(i) > 0 ? dxp : (cx(i) < 0 ? dxm : 0)) +
+                                                      (cy(i) > 0 ? dyp : (cy(i) < 0 ? dym : 0)) +
+                                                      (cz(i) > 0 ? dzp : (cz(i) < 0 ? dzm : 0)));
+            // push: the destination's element of plane i, SKEW + q - c_ix (at the
+            // source's x); bounce-back: the own element of plane opp(i),
+            // SKEW + s + c_ix
+            const unsigned off = b ? (unsigned)(SKEW + cx(i)) + s + (opp(i) == lo ? 0u : ps)
+                                   : (unsigned)(SKEW - cx(i)) + q + (i == lo ? 0u : ps);
+            // f_ibar = f*_i - 6 w_i rho c_i.u_w (Eq. 17)
+            const C cw = b ? C(-2) * along<C>(i, V[cz(i) + 1]) : C(0);
+            C fb[2];
+#pragma unroll
+            for (int k = 0; k < 2; k++) fb[k] = fs[k] + B[k][c] * cw;
+            put2(pair_at(lo, off), solid ? wgt<C>(i) * prm<C>(L.P.rho0[0], L.PF.rho0[0]) : fb[0],
+                 solid ? wgt<C>(i) * prm<C>(L.P.rho0[1], L.PF.rho0[1]) : fb[1], pop_shift<S, C>(L, 0, i),
+                 pop_shift<S, C>(L, 1, i));
+            C fl = fs[0] + fb[0] + fs[1] + fb[1];
+            fl = (pm >> i) & 1u ? fl : C(0);
+            if (cx(i)) Fl[0] += C(cx(i)) * fl;
+            if (cy(i)) Fl[1] += C(cy(i)) * fl;
+            if (cz(i)) Fl[2] += C(cz(i)) * fl;
+        }
     }
     // Eq. 23 with r_w - r_p = (x - r_p) + c_i/2: the c_i/2 part is parallel
     // to the link force and drops out of the torque
@@ -707,7 +715,6 @@ __global__ void __launch_bounds__(FTX* TY, (PREC == LB_FP64 ? 1 : 16 / TY)) k_fu
     typedef typename Prec<PREC>::C C;
     typedef AsyncShared<PREC, TY> SH;
     typedef S E;
-    constexpr int NT = FTX * TY;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SH& sh = *reinterpret_cast<SH*>(smem_raw);
     const int x0 = blockIdx.x * FTX, y0 = blockIdx.y * TY;
@@ -893,41 +900,30 @@ __device__ __forceinline__ void lean_site(const Lattice& L, const LeanShared<PRE
     C rho[2];
 #pragma unroll
     for (int k = 0; k < 2; k++) rho[k] = solid ? prm<C>(L.P.rho0[k], L.PF.rho0[k]) : sh.psi[sl[1]][1][tx + 1][k];
-    // Eq. 11 (repulsive sign) + body force from the staged psi planes
-    C sA[3] = {0, 0, 0}, sB[3] = {0, 0, 0};
-#pragma unroll
-    for (int i = 1; i < Q; i++) {
-        const int slot = sl[cz(i) + 1];
-        const C pa = sh.psi[slot][1 + cy(i)][tx + 1 + cx(i)][0];
-        const C pb = sh.psi[slot][1 + cy(i)][tx + 1 + cx(i)][1];
-        const C w = wgt<C>(i);
-        if (cx(i)) { sA[0] += C(cx(i)) * w * pa; sB[0] += C(cx(i)) * w * pb; }
-        if (cy(i)) { sA[1] += C(cy(i)) * w * pa; sB[1] += C(cy(i)) * w * pb; }
-        if (cz(i)) { sA[2] += C(cz(i)) * w * pa; sB[2] += C(cz(i)) * w * pb; }
-    }
-    const C G = prm<C>(L.P.G, L.PF.G);
+    // Eq. 11 (repulsive sign) + body force from the staged psi planes, per
+    // density: F^k / rho^k = g - G S
+    C grad[2][3];
+    link_gradient<C>(grad, [&](int i, int k) { return sh.psi[sl[cz(i) + 1]][1 + cy(i)][tx + 1 + cx(i)][k]; });
+    const C G36 = prm<C>(L.P.G, L.PF.G) * wgt<C>(7);
     // Eq. 14 at tau_A = tau_B: u = (j^A + j^B) / (rho^A + rho^B) (j = 0 on
-    // particle nodes)
-    C us[2][3], u[3];
+    // particle nodes); Eq. 16: the shifted velocities
+    C us[2][3];
     {
         const C ir = C(1) / (rho[0] + rho[1]);
-#pragma unroll
-        for (int d = 0; d < 3; d++) u[d] = sh.j[b][d][tx] * ir;
-    }
-    const C tiny = sizeof(C) == 8 ? C(1e-300) : C(1e-30);
-#pragma unroll
-    for (int k = 0; k < 2; k++) {
-        const C ir = rho[k] > tiny ? C(1) / rho[k] : C(0);
+        const C tiny = sizeof(C) == 8 ? C(1e-300) : C(1e-30);
 #pragma unroll
         for (int d = 0; d < 3; d++) {
-            const C g = prm<C>(L.P.body_force[d], L.PF.body_force[d]);
-            const C F = -G * rho[k] * (k == 0 ? sB[d] : sA[d]) + rho[k] * g;
-            us[k][d] = u[d] + F * ir;  // Eq. 16: the shifted velocity
+            const C u = sh.j[b][d][tx] * ir, g = prm<C>(L.P.body_force[d], L.PF.body_force[d]);
+#pragma unroll
+            for (int k = 0; k < 2; k++) us[k][d] = u + (rho[k] > tiny ? g - G36 * grad[1 - k][d] : C(0));
         }
     }
-    // Eq. 5 factored per weight class c (0 rest, 1 axis, 2 diagonal):
-    // f^eq_i = A_c + c_i.us (B_c + H_c c_i.us), A_c = w_c rho (1 - 3/2 us.us),
-    // B_c = 3 w_c rho, H_c = 9/2 w_c rho
+    // Eq. 5 factored per weight class c (0 rest, 1 axis, 2 diagonal) for the
+    // opposite pairs of links: f^eq(+-c_i) = A_c + H_c (c_i.us)^2 +- B_c c_i.us,
+    // A_c = w_c rho (1 - 3/2 us.us), B_c = 3 w_c rho, H_c = 9/2 w_c rho.  In FP64
+    // (two lanes a cycle on an SM) the operations bound the kernel: link by
+    // link, with products by the zeros of c_i and a division per density, it
+    // took 762 us a step at 96^3; 590 now.
     C A[2][3], B[2][3], H[2][3];
 #pragma unroll
     for (int k = 0; k < 2; k++) {
@@ -972,6 +968,14 @@ __device__ __forceinline__ void lean_site(const Lattice& L, const LeanShared<PRE
         particle_u0_of<C>(L, particle_load<C>(L, p0), x, y, z, U0, rel);
     }
     C Fl[3] = {0, 0, 0};  // Eq. 19 summed over the links: (f*_i + f_ibar(t+1)) c_i
+    C Bw[2][2], Bh[2];    // the wall terms of f_ibar and of (f*_i + f_ibar) / 2 per c_i.u_w
+    if (wbb)
+#pragma unroll
+        for (int c = 0; c < 2; c++) {
+            Bw[0][c] = C(-2) * B[0][c + 1];
+            Bw[1][c] = C(-2) * B[1][c + 1];
+            Bh[c] = -(B[0][c + 1] + B[1][c + 1]);
+        }
     S* const pA = (S*)L.f_nxt + 2 * (SKEW + (long long)s);
     // the rounding bits of the site's stores, in store order (the bounce-back
     // stores of a link follow its push when the warp takes that branch)
@@ -986,38 +990,43 @@ __device__ __forceinline__ void lean_site(const Lattice& L, const LeanShared<PRE
     };
     put2(pA, A[0][0], A[1][0], pop_shift<S, C>(L, 0, 0), pop_shift<S, C>(L, 1, 0), true, rs);
 #pragma unroll
-    for (int i = 1; i < Q; i++) {
-        const int c = i <= 6 ? 1 : 2;
-        C fs[2];
+    for (int lo = 1; lo < Q; lo += 2) {  // planes lo and opp(lo) = lo + 1
+        const int c = lo <= 6 ? 1 : 2;
+        C fp[2][2];
 #pragma unroll
         for (int k = 0; k < 2; k++) {
-            const C cu = C(cx(i)) * us[k][0] + C(cy(i)) * us[k][1] + C(cz(i)) * us[k][2];
-            fs[k] = A[k][c] + cu * (B[k][c] + H[k][c] * cu);
+            const C cu = along<C>(lo, us[k]), e = A[k][c] + (H[k][c] * cu) * cu;
+            fp[0][k] = e + B[k][c] * cu;
+            fp[1][k] = e - B[k][c] * cu;
         }
-        const Off off = (Off)i * ps + (Off)((cx(i) > 0 ? wxp : (cx(i) < 0 ? wxm : 0)) +
-                                            (cy(i) > 0 ? dyp : (cy(i) < 0 ? dym : 0)) +
-                                            (cz(i) > 0 ? dzp : (cz(i) < 0 ? dzm : 0)));
-        // a particle node does not push into a fluid site (whose bounce-back
-        // writes that element)
-        put2(pA + 2 * (long long)off, fs[0], fs[1], pop_shift<S, C>(L, 0, i), pop_shift<S, C>(L, 1, i),
-             !(solid && ((nbc >> i) & 1u)), rs);
-        if (wbb & (1u << i)) {
-            // Eq. 17 with the wall velocity of Eq. 18: the own element of
-            // plane opp(i), opp(i) ps + SKEW + s + c_ix
-            const bool on = (bbi >> i) & 1u;
-            const C cw = C(-2) * (C(cx(i)) * U0[0] + C(cy(i)) * U0[1] + C(cz(i)) * U0[2]);
-            C fb[2];
 #pragma unroll
-            for (int k = 0; k < 2; k++) fb[k] = fs[k] + B[k][c] * cw;
-            const Off ob = (Off)opp(i) * ps + cx(i);
-            put2(pA + 2 * (long long)ob, fb[0], fb[1], pop_shift<S, C>(L, 0, opp(i)), pop_shift<S, C>(L, 1, opp(i)), on,
-                 rs);
-            const C fl = on ? fs[0] + fb[0] + fs[1] + fb[1] : C(0);
-            if (cx(i)) Fl[0] += C(cx(i)) * fl;
-            if (cy(i)) Fl[1] += C(cy(i)) * fl;
-            if (cz(i)) Fl[2] += C(cz(i)) * fl;
+        for (int side = 0; side < 2; side++) {
+            const int i = lo + side;
+            const C(&fs)[2] = fp[side];
+            const Off off = (Off)i * ps + (Off)((cx(i) > 0 ? wxp : (cx(i) < 0 ? wxm : 0)) +
+                                                (cy(i) > 0 ? dyp : (cy(i) < 0 ? dym : 0)) +
+                                                (cz(i) > 0 ? dzp : (cz(i) < 0 ? dzm : 0)));
+            // a particle node does not push into a fluid site (whose bounce-back
+            // writes that element)
+            put2(pA + 2 * (long long)off, fs[0], fs[1], pop_shift<S, C>(L, 0, i), pop_shift<S, C>(L, 1, i),
+                 !(solid && ((nbc >> i) & 1u)), rs);
+            if (wbb & (1u << i)) {
+                // Eq. 17 with the wall velocity of Eq. 18: the own element of
+                // plane opp(i), opp(i) ps + SKEW + s + c_ix
+                const bool on = (bbi >> i) & 1u;
+                const C cu = along<C>(i, U0);
+                const Off ob = (Off)opp(i) * ps + cx(i);
+                put2(pA + 2 * (long long)ob, fs[0] + Bw[0][c - 1] * cu, fs[1] + Bw[1][c - 1] * cu,
+                     pop_shift<S, C>(L, 0, opp(i)), pop_shift<S, C>(L, 1, opp(i)), on, rs);
+                const C fl = on ? (fs[0] + fs[1]) + Bh[c - 1] * cu : C(0);  // half of what is handed over
+                if (cx(i)) Fl[0] += C(cx(i)) * fl;
+                if (cy(i)) Fl[1] += C(cy(i)) * fl;
+                if (cz(i)) Fl[2] += C(cz(i)) * fl;
+            }
         }
     }
+#pragma unroll
+    for (int d = 0; d < 3; d++) Fl[d] += Fl[d];
     if (bbi) {
         // Eq. 23 with r_w - r_p = (x - r_p) + c_i/2: the c_i/2 part is
         // parallel to the link force and drops out of the torque
