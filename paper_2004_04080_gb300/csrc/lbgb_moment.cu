@@ -66,12 +66,12 @@ __device__ __forceinline__ F2 f2(float x, float y) {
 }
 __device__ __forceinline__ F2 f2(float x) { return f2(x, x); }
 __device__ __forceinline__ float lo(F2 a) {
-    float x, y;
+    [[maybe_unused]] float x, y;
     asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(a.v));
     return x;
 }
 __device__ __forceinline__ float hi(F2 a) {
-    float x, y;
+    [[maybe_unused]] float x, y;
     asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(a.v));
     return y;
 }
@@ -691,24 +691,25 @@ __global__ void __launch_bounds__(MNT, NK == 1 ? 4 : 3)
 }
 
 // The bounce-back links of the listed boundary sites (`parts` blocks per
-// segment of the grid of k_moments): the values that come back (Eqs. 17, 18) added to the
-// sums k_moments left in psi_o, mom_o, and the forces and torques they hand to
-// the particles (Eqs. 19, 22, 23).  A kernel of its own: a site's particle is
-// two dependent loads away, which inside the march of k_moments every plane of
-// a block waited for (256^3, 2407 particles: 654 us together, 366 + 128 us
-// apart).  It is bound by the latency of those loads.  The sites of a warp mostly belong to a few particles
-// in runs: the fixed-point words of a run are summed across the lanes and
-// added once (integer sums: the bits do not depend on the grouping).
+// segment of the grid of k_moments): the values that come back (Eqs. 17, 18)
+// added to the sums k_moments left in psi_o, mom_o, and the forces and torques
+// they hand to the particles (Eqs. 19, 22, 23).  A kernel of its own: a site's
+// particle is two dependent loads away, which inside the march of k_moments
+// every plane of a block waited for (256^3, 2407 particles: 654 us together, 366
+// + 128 us apart; at the end of each block, 15 warps on an SM, 512 x 512 x 256
+// took 1994 us instead of 1286 + 474).  It is bound by the latency of those
+// loads: the sums are fetched beside them, and the links of a site are
+// evaluated by opposite pairs without branches (103 -> 88 us at 256^3).  The
+// sites of a warp mostly belong to a few particles in runs: the fixed-point
+// words of a run are summed across the lanes and added once (integer sums: the
+// bits do not depend on the grouping).
 __global__ void __launch_bounds__(128) k_bounce_links(const __grid_constant__ Lattice L, float* __restrict__ psi_o,
                                                        float* __restrict__ mom_o, LinkList list, int zc, int TW,
-                                                       int parts) {
+                                                       int parts, long long unit) {
     const int bx = blockIdx.x / parts, z0 = blockIdx.z * zc, x0 = bx * TW, y0 = blockIdx.y * MROWS;
     const int n = list.count[bx + gridDim.x / parts * (blockIdx.y + gridDim.y * blockIdx.z)];
     const unsigned* seg = list.rec + segment_of(L, x0, y0, min(MROWS, L.ny - y0), z0, min(zc, L.nz - z0));
     const int lane = threadIdx.x & 31, nx = L.nx, nxy = L.nx * L.ny;
-    // what a link of weight 1/36 of the reference fluid hands over (2 f*_i of
-    // both components), in fixed point
-    const long long unit = __double2ll_rn(((double)L.rref[0] + (double)L.rref[1]) * (2.0 / 36.0 * 1099511627776.0));
     for (int k0 = (int)(blockIdx.x % parts * 128 + threadIdx.x) - lane; k0 < n; k0 += 128 * parts) {
         const int k = k0 + lane;
         int p = -1, exact[3] = {0, 0, 0};
@@ -725,6 +726,12 @@ __global__ void __launch_bounds__(128) k_bounce_links(const __grid_constant__ La
             }
             const float ra = __uint_as_float(get());
             r = f2(ra, __uint_as_float(get()));
+            // the sums that the links are added to, on their way while the
+            // particle is looked up
+            F2* ps = reinterpret_cast<F2*>(psi_o) + s;
+            float* mo = mom_o + s;
+            const F2 sum = *ps;
+            const float js[3] = {mo[0], mo[L.pstride], mo[2 * L.pstride]};
             const int z = (int)(s / (unsigned)nxy), yx = (int)(s - (unsigned)z * (unsigned)nxy), y = yx / nx, x = yx - y * nx;
             const int dxp = x == nx - 1 ? 1 - nx : 1, dxm = x == 0 ? nx - 1 : -1;
             const int dyp = y == L.ny - 1 ? nx - nxy : nx, dym = y == 0 ? nxy - nx : -nx;
@@ -785,21 +792,32 @@ __global__ void __launch_bounds__(128) k_bounce_links(const __grid_constant__ La
             } else {
                 p = owner_of(__ffs(bits) - 1);
                 particle_u0<float>(L, p, x, y, z, U, rel);
+                const float V[3] = {-6.f * U[0], -6.f * U[1], -6.f * U[2]};
+                // the opposite links of a pair hand over e + q, e - q and get back
+                // e + o, e - o; those the site has count by the sum and the
+                // difference of their bits: no branch (half of the lanes of a warp
+                // have a given link, so branches ran for all of them)
 #pragma unroll
-                for (int i = 1; i < Q; i++) {
-                    if (!((bits >> i) & 1u)) continue;
+                for (int i = 1; i < Q; i += 2) {
+                    const float up = (bits >> i) & 1u ? 1.f : 0.f, dn = (bits >> (i + 1)) & 1u ? 1.f : 0.f;
+                    const float m = up + dn, df = up - dn;
                     F2 ch = f2(0.f);
-                    float cu = 0;
+                    bool any = false;
 #pragma unroll
                     for (int d = 0; d < 3; d++) {
                         const int c = d == 0 ? cx(i) : (d == 1 ? cy(i) : cz(i));
-                        if (c > 0) ch = ch + h[d], cu += U[d];
-                        if (c < 0) ch = ch - h[d], cu -= U[d];
+                        if (c == 0) continue;
+                        ch = !any ? (c > 0 ? h[d] : f2(0.f) - h[d]) : (c > 0 ? ch + h[d] : ch - h[d]);
+                        any = true;
                     }
-                    const float fl = link(i, ch, cu, cx(i), cy(i), cz(i));
-                    F[0] += cx(i) * fl;
-                    F[1] += cy(i) * fl;
-                    F[2] += cz(i) * fl;
+                    const F2 q = (i <= 6 ? r4 : r2) * ch, e = fma2(q, ch, i <= 6 ? P2 : P);
+                    const F2 o = fma2(i <= 6 ? r2 : r, f2(along<float>(i, V)), q);
+                    back = fma2(f2(m), e, fma2(f2(df), o, back));
+                    const float es = df * (lo(e) + hi(e)), os = lo(o) + hi(o), qs = lo(q) + hi(q);
+                    const float jb = fmaf(m, os, es), fl = jb + fmaf(m, qs, es);
+                    if (cx(i)) j[0] -= cx(i) * jb, F[0] += cx(i) * fl;
+                    if (cy(i)) j[1] -= cy(i) * jb, F[1] += cy(i) * fl;
+                    if (cz(i)) j[2] -= cz(i) * jb, F[2] += cz(i) * fl;
                 }
                 // Eq. 23 with r_w - r_p = (x - r_p) + c_i/2: the c_i/2 part is
                 // parallel to the link force and drops out of the torque
@@ -817,12 +835,10 @@ __global__ void __launch_bounds__(128) k_bounce_links(const __grid_constant__ La
             back = fma2(f2(nw), ref, back);
 #pragma unroll
             for (int d = 0; d < 3; d++) j[d] = fmaf((float)-nd[d], rr, j[d]);
-            F2* ps = reinterpret_cast<F2*>(psi_o) + s;
             constexpr float h36 = 1.0f / 36.0f, l36 = (float)(1.0 / 36.0 - (double)h36);
-            *ps = fma2(back, f2(h36), fma2(back, f2(l36), *ps));
-            float* mo = mom_o + s;
+            *ps = fma2(back, f2(h36), fma2(back, f2(l36), sum));
 #pragma unroll
-            for (int d = 0; d < 3; d++) *mo = fmaf(j[d], h36, fmaf(j[d], l36, *mo)), mo += L.pstride;
+            for (int d = 0; d < 3; d++) *mo = fmaf(j[d], h36, fmaf(j[d], l36, js[d])), mo += L.pstride;
         }
         add_runs(L, ACC_FLIQ, p, F, T, exact, unit);
     }
@@ -944,7 +960,10 @@ static int launch_moments_t(const Lattice& L, void* psi_o, void* mom_o, cudaStre
         // about a fifth of the sites are boundary sites in a dense suspension:
         // blocks for two or three rounds over a segment
         const int parts = (zc * TW * MROWS + 128 * 16 - 1) / (128 * 16);
-        k_bounce_links<<<dim3(gx * parts, gy, grid.z), 128, 0, st>>>(L, po, mo, list, zc, TW, parts);
+        // what a link of weight 1/36 of the reference fluid hands over (2 f*_i of
+        // both components), in fixed point
+        const long long unit = llrint(((double)L.rref[0] + (double)L.rref[1]) * (2.0 / 36.0 * 1099511627776.0));
+        k_bounce_links<<<dim3(gx * parts, gy, grid.z), 128, 0, st>>>(L, po, mo, list, zc, TW, parts, unit);
         n++;
     }
     if (!L.per[2]) {
