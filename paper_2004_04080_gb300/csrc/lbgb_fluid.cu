@@ -833,7 +833,7 @@ __global__ void __launch_bounds__(FTX* TY, (PREC == LB_FP64 ? 1 : 16 / TY)) k_fu
     cp_async_wait_all();
 }
 
-static int z_chunks(const Lattice& L, int tiles, int per_sm, int zmin);
+static int z_chunks(const Lattice& L, int tiles, int per_sm, int zmin, int zlow, int waves);
 
 constexpr int WNSLOT = 5;  // psi planes a lean warp holds: z-1 .. z+3
 constexpr int WPB = 4;     // warps (rows) per block of the lean kernel
@@ -1177,7 +1177,11 @@ static int launch_lean_t(const Lattice& L, cudaStream_t st) {
     const size_t smem = sizeof(LeanShared<P>) * WPB;
     const int per_sm = kernel_setup<k_lean<P, SR, NEAR>>(FTX * WPB, smem);
     int tiles = ((L.nx + FTX - 1) / FTX) * ((L.ny + WPB - 1) / WPB);
-    int zc = z_chunks(L, tiles, per_sm, 8);
+    // short marches where 8 planes leave SMs idle or unevenly loaded, in FP64
+    // above all (a block keeps its SM's two FP64 lanes busy by itself): a step at
+    // 32^3 FP64 155 -> 92 us, 96^3 FP64 898 -> 825, one step of 32^3 FP32 92 -> 84;
+    // at 256^3 FP32 marches below 4 planes are the slower ones (956 against 914)
+    int zc = z_chunks(L, tiles, per_sm, 8, 2, P == LB_FP64 ? 8 : 2);
     dim3 grid((L.nx + FTX - 1) / FTX, (L.ny + WPB - 1) / WPB, (L.nz + zc - 1) / zc);
     k_lean<P, SR, NEAR><<<grid, dim3(FTX, WPB), smem, st>>>(L, zc);
     return 1;
@@ -1469,8 +1473,9 @@ int launch_wall_psi(const Lattice& L, int prec, cudaStream_t st) {
 
 // Number of z chunks for a kernel with `per_sm` resident blocks per SM: the
 // grid (tiles x chunks) is close to a whole number of full waves, with
-// chunks of at least `zmin` planes.
-static int z_chunks(const Lattice& L, int tiles, int per_sm, int zmin) {
+// chunks of at least `zmin` planes; where that gives fewer than four waves, chunks
+// of `zmin` planes, or fewer (at least `zlow`) until the blocks make `waves` waves.
+static int z_chunks(const Lattice& L, int tiles, int per_sm, int zmin, int zlow, int waves) {
     long long R = (long long)device_sms() * per_sm;
     int best = 1;
     double best_eff = 0;
@@ -1484,7 +1489,11 @@ static int z_chunks(const Lattice& L, int tiles, int per_sm, int zmin) {
         if (best_eff >= 0.98) break;
         if (zc <= 1) break;
     }
-    if (best_eff == 0) best = zmin < L.nz ? zmin : L.nz;
+    if (best_eff == 0) {
+        // too few blocks for that: down to zlow planes, until they make `waves`
+        best = zmin < L.nz ? zmin : L.nz;
+        while (best > zlow && (long long)tiles * ((L.nz + best - 1) / best) < waves * R) best--;
+    }
     return best;
 }
 
@@ -1495,7 +1504,7 @@ static int launch_fused_async_t(const Lattice& L, cudaStream_t st) {
     const size_t smem = sizeof(SH);
     const int per_sm = kernel_setup<k_fused_async<P, TY, SR>>(NT, smem);
     int tiles = ((L.nx + FTX - 1) / FTX) * ((L.ny + TY - 1) / TY);
-    int zc = z_chunks(L, tiles, per_sm, 8);
+    int zc = z_chunks(L, tiles, per_sm, 8, 8, 1);
     dim3 grid((L.nx + FTX - 1) / FTX, (L.ny + TY - 1) / TY, (L.nz + zc - 1) / zc);
     k_fused_async<P, TY, SR><<<grid, dim3(FTX, TY), smem, st>>>(L, zc);
     return 1;

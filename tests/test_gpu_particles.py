@@ -3,7 +3,7 @@ import numpy as np
 import pytest
 
 from paper_2004_04080_gb300.workloads import mixture_densities
-from test_gpu_parity import compare_fields, run_both
+from test_gpu_parity import compare_colloids, compare_fields, run_both
 
 pytestmark = pytest.mark.gpu
 
@@ -67,3 +67,21 @@ def test_overlap_is_reported_by_every_call(prec):
     for _ in range(2):
         with pytest.raises(LBError):
             g.step(1)
+
+
+@pytest.mark.parametrize("prec,tol", [("fp64", 1e-12), ("fp32", 1e-5)])
+@pytest.mark.parametrize("walls", [False, True])
+@pytest.mark.parametrize("shape", [(12, 12, 11), (32, 13, 12), (36, 12, 13), (32, 40, 33)])
+def test_lean_short_marches(shape, walls, prec, tol):
+    """Calls of one step on lattices whose lean kernel takes marches of two or
+    a few planes, of which the last may be shorter, with a particle across
+    several of them.  Bounds of the forms."""
+    col = dict(pos=[[s / 2 + 0.3 for s in shape]], radius=[2.7], mass=[300.0], vel=[[0.03, -0.02, 0.01]],
+               omega=[[0.0, 0.01, 0.02]])
+    params = dict(G=0.4, zeta=(0.05, -0.05), bc=(1, 1, 0 if walls else 1))
+    g, o = run_both(shape, params, 1, prec, col, mixture_densities(shape, seed=9, amp=0.05))
+    for _ in range(5):
+        g.step(1)
+        o.step(1)
+    compare_fields(g, o, tol)
+    compare_colloids(g, o, tol)
