@@ -42,13 +42,6 @@ struct AdjArgs {
     double* red;          // block partials [blocks][ADJ_VALUES][2]
 };
 
-// E_i(rho, u) / rho = w_i (1 + 3 c.u + 9/2 (c.u)^2 - 3/2 u.u)
-template <typename C>
-__device__ __forceinline__ C eq_shape(int i, C ux, C uy, C uz, C uu) {
-    C cu = C(cx(i)) * ux + C(cy(i)) * uy + C(cz(i)) * uz;
-    return wgt<C>(i) * (C(1) + C(3) * cu + C(4.5) * cu * cu - C(1.5) * uu);
-}
-
 // weighted moments of an adjoint vector mu over the lattice:
 // m0 = sum w mu, m1 = sum w mu c, m2 = sum w mu c c^T (xx, yy, zz, xy, xz, yz)
 template <typename C>
@@ -58,16 +51,38 @@ struct Mom {
 
 template <typename C>
 __device__ __forceinline__ void moments_of(const C (&mu)[Q], Mom<C>& M) {
-    M.m0 = 0;
-    for (int d = 0; d < 3; d++) M.m1[d] = 0;
-    for (int d = 0; d < 6; d++) M.m2[d] = 0;
+    // by opposite pairs, no products by the zeros of c_i: 60 operations (200
+    // link by link)
+    C ax = 0, dg = 0, sd[6] = {0, 0, 0, 0, 0, 0}, sa[3], da[3], dd[3] = {0, 0, 0};
 #pragma unroll
-    for (int i = 0; i < Q; i++) {
-        C wm = wgt<C>(i) * mu[i];
-        M.m0 += wm;
-        M.m1[0] += C(cx(i)) * wm; M.m1[1] += C(cy(i)) * wm; M.m1[2] += C(cz(i)) * wm;
-        M.m2[0] += C(cx(i) * cx(i)) * wm; M.m2[1] += C(cy(i) * cy(i)) * wm; M.m2[2] += C(cz(i) * cz(i)) * wm;
-        M.m2[3] += C(cx(i) * cy(i)) * wm; M.m2[4] += C(cx(i) * cz(i)) * wm; M.m2[5] += C(cy(i) * cz(i)) * wm;
+    for (int i = 1; i < Q; i += 2) {  // opp(i) = i + 1
+        const C sum = mu[i] + mu[i + 1], dif = mu[i] - mu[i + 1];
+        const int c[3] = {cx(i), cy(i), cz(i)};
+        if (i <= 6) {
+            ax += sum;
+            const int d = c[0] ? 0 : (c[1] ? 1 : 2);
+            sa[d] = sum;
+            da[d] = c[d] > 0 ? dif : -dif;
+            continue;
+        }
+        dg += sum;
+#pragma unroll
+        for (int d = 0; d < 3; d++) {
+            if (c[d] > 0) dd[d] += dif;
+            if (c[d] < 0) dd[d] -= dif;
+            if (c[d] != 0) sd[d] += sum;
+        }
+        const int q = c[2] == 0 ? 3 : (c[1] == 0 ? 4 : 5);  // xy, xz, yz
+        const int sign = (c[0] ? c[0] : c[1]) * (c[2] ? c[2] : c[1]);
+        if (sign > 0) sd[q] += sum; else sd[q] -= sum;
+    }
+    const C w0 = wgt<C>(0), w1 = wgt<C>(1), w2 = wgt<C>(7);
+    M.m0 = w0 * mu[0] + (w1 * ax + w2 * dg);
+#pragma unroll
+    for (int d = 0; d < 3; d++) {
+        M.m1[d] = w1 * da[d] + w2 * dd[d];
+        M.m2[d] = w1 * sa[d] + w2 * sd[d];
+        M.m2[3 + d] = w2 * sd[3 + d];
     }
 }
 
@@ -91,108 +106,115 @@ __device__ __forceinline__ void mom_grad(const Mom<C>& M, const C (&u)[3], C (&g
     g[2] = C(3) * M.m1[2] + C(9) * m2u2 - C(3) * u[2] * M.m0;
 }
 
-// sum over the block of one double per thread, written by thread 0 to *out
-// (warp shuffles, then warps in order; blockDim.x a multiple of 32)
-__device__ void block_sum_store(double v, double* out) {
-    __shared__ double sh[32];
-    int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
+// sums over the block of NV doubles per thread, thread 0 writing value v to
+// out[v * stride] (warp shuffles, then warps in order; blockDim.x a multiple of 32)
+template <int NV>
+__device__ __forceinline__ void block_sum_store(double (&v)[NV], double* out, long long stride) {
+    __shared__ double sh[NV][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int m = 0; m < NV; m++)
+        for (int off = 16; off > 0; off >>= 1) v[m] += __shfl_down_sync(0xffffffffu, v[m], off);
+    if (lane == 0)
+#pragma unroll
+        for (int m = 0; m < NV; m++) sh[m][warp] = v[m];
     __syncthreads();
-    if (lane == 0) sh[warp] = v;
-    __syncthreads();
-    if (threadIdx.x == 0) {
+    if (threadIdx.x < NV) {
         double t = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); w++) t += sh[w];
-        *out = t;
+        for (int w = 0; w < (int)(blockDim.x >> 5); w++) t += sh[threadIdx.x][w];
+        out[threadIdx.x * stride] = t;
     }
 }
 
 // Local adjoint of the collision and streaming at each fluid site.
 template <int PREC>
-__global__ void __launch_bounds__(128) k_adj_local(Lattice L, AdjArgs A) {
+__global__ void __launch_bounds__(128, (PREC == LB_FP64 ? 2 : 4)) k_adj_local(Lattice L, AdjArgs A) {
     typedef typename Prec<PREC>::S S;
     typedef typename Prec<PREC>::C C;
     int x = blockIdx.x * blockDim.x + threadIdx.x;
     int y = blockIdx.y, z = blockIdx.z;
-    C part[ADJ_VALUES] = {0, 0, 0, 0, 0};
+    C part[3] = {0, 0, 0};
     long long s = (long long)x + (long long)L.nx * ((long long)y + (long long)L.ny * z);
     const C* Lin = (const C*)A.adj_in;
     const C* Rin = Lin + 2 * Q * L.pstride;
     C* Lout = (C*)A.adj_out;
     C* sb = (C*)A.sbar;
-    bool act = x < L.nx && !L.mask[s];
-    if (act) {
+    const uint32_t nbc = x < L.nx ? L.nb[s] : NB_SOLID;
+    if (!(nbc & NB_SOLID)) {
         SiteNbr n = site_nbr(L, x, y, z);
-        C fv[2][Q], rho[2], j[2][3], F[2][3], u[3], om;
+        C fv[2][Q], rho[2], j[2][3], u[3], om;
         load_site<PREC>(L, (const S*)L.f_cur, s, fv, rho, j);
-        // S^A, S^B (the force uses S of the other component)
-        C SA[3] = {0, 0, 0}, SB[3] = {0, 0, 0};
+        // F^A / rho^A = g - G S^B and F^B / rho^B = g - G S^A (acc), 36 S in grad
+        C grad[2][3], acc[2][3];
         {
             const C* psi = (const C*)L.psi;
             const C* pw = (const C*)L.psi_wall;
-            long long nxy = (long long)L.nx * L.ny;
+            const long long nxy = (long long)L.nx * L.ny;
+            C ps[Q][2];
 #pragma unroll
             for (int i = 1; i < Q; i++) {
-                C pa, pb;
+                const C* q = psi;
+                long long m;
                 if (nbr_is_wall(n, i)) {
-                    int X = cx(i) == 0 ? n.x : (cx(i) > 0 ? n.xp : n.xm);
-                    int Y = cy(i) == 0 ? n.y : (cy(i) > 0 ? n.yp : n.ym);
-                    int side = cz(i) < 0 ? 0 : 1;
-                    long long w = (long long)X + (long long)L.nx * Y;
-                    pa = pw[2 * (side * nxy + w)];
-                    pb = pw[2 * (side * nxy + w) + 1];
+                    const int X = cx(i) == 0 ? n.x : (cx(i) > 0 ? n.xp : n.xm);
+                    const int Y = cy(i) == 0 ? n.y : (cy(i) > 0 ? n.yp : n.ym);
+                    q = pw;
+                    m = (cz(i) < 0 ? 0 : nxy) + (long long)X + (long long)L.nx * Y;
                 } else {
-                    long long m = nbr_index(L, n, i);
-                    pa = psi[2 * m];
-                    pb = psi[2 * m + 1];
+                    m = nbr_index(L, n, i);
                 }
-                C w = wgt<C>(i);
-                SA[0] += C(cx(i)) * w * pa; SA[1] += C(cy(i)) * w * pa; SA[2] += C(cz(i)) * w * pa;
-                SB[0] += C(cx(i)) * w * pb; SB[1] += C(cy(i)) * w * pb; SB[2] += C(cz(i)) * w * pb;
+                ps[i][0] = q[2 * m];
+                ps[i][1] = q[2 * m + 1];
             }
+            link_gradient<C>(grad, [&](int i, int k) { return ps[i][k]; });
         }
-        C G = C(L.P.G);
-        for (int d = 0; d < 3; d++) {
-            C g = C(L.P.body_force[d]);
-            F[0][d] = -G * rho[0] * SB[d] + rho[0] * g;
-            F[1][d] = -G * rho[1] * SA[d] + rho[1] * g;
-        }
+        const C G = prm<C>(L.P.G, L.PF.G), G36 = G * wgt<C>(7);
         mixture<C>(L, rho, j, u, om);
-        C tiny = sizeof(C) == 8 ? C(1e-300) : C(1e-30);
+        const C tiny = sizeof(C) == 8 ? C(1e-300) : C(1e-30);
         C v[2][3];
+#pragma unroll
         for (int k = 0; k < 2; k++)
-            for (int d = 0; d < 3; d++) v[k][d] = rho[k] > tiny ? u[d] + F[k][d] / rho[k] : u[d];
+#pragma unroll
+            for (int d = 0; d < 3; d++) {
+                acc[k][d] = prm<C>(L.P.body_force[d], L.PF.body_force[d]) - G36 * grad[1 - k][d];
+                v[k][d] = rho[k] > tiny ? u[d] + acc[k][d] : u[d];
+            }
         C a = C(1) - om;
         // incoming adjoint mu = dJ/df*, and the wall bounce-back density term
         C mu[2][Q];
         C rbar[2] = {0, 0};
         const double* uwlo = L.P.wall_u_lo;
         const double* uwhi = L.P.wall_u_hi;
+        // the population of the neighbour, or, of a link into a wall or a fixed
+        // particle, the site's own one of the opposite link: the class bits
+        // pick the address, so that all loads are under way together (a branch
+        // per link on the neighbour's mask took the loads one after the other:
+        // 96 -> 47 us at 64^3)
 #pragma unroll
         for (int i = 0; i < Q; i++) {
-            if (i != 0 && nbr_is_wall(n, i)) {
+            const bool wall = i != 0 && nbr_is_wall(n, i), own = i == 0 || wall || ((nbc >> i) & 1u);
+            const long long m = own ? s : nbr_index(L, n, i);
+            const long long e = (own ? opp(i) : i) * L.pstride + m;
+#pragma unroll
+            for (int k = 0; k < 2; k++) mu[k][i] = Lin[k * Q * L.pstride + e] + Rin[k * L.pstride + m];
+        }
+        if (n.wall_lo || n.wall_hi) {
+#pragma unroll
+            for (int i = 1; i < Q; i++) {
+                if (cz(i) == 0 || !nbr_is_wall(n, i)) continue;
                 const double* uw = cz(i) < 0 ? uwlo : uwhi;
-                C cu = C(cx(i) * uw[0] + cy(i) * uw[1] + cz(i) * uw[2]);
-                for (int k = 0; k < 2; k++) {
-                    C lam = Lin[((long long)(k * Q + opp(i))) * L.pstride + s] + Rin[k * L.pstride + s];
-                    mu[k][i] = lam;
-                    rbar[k] += lam * (-C(6) * wgt<C>(i) * cu);
-                }
-                continue;
+                const C cu = C(cx(i) * uw[0] + cy(i) * uw[1] + cz(i) * uw[2]);
+                for (int k = 0; k < 2; k++) rbar[k] += mu[k][i] * (-C(6) * wgt<C>(i) * cu);
             }
-            long long m = i == 0 ? s : nbr_index(L, n, i);
-            if (i == 0 || !L.mask[m]) {
-                for (int k = 0; k < 2; k++)
-                    mu[k][i] = Lin[((long long)(k * Q + i)) * L.pstride + m] + Rin[k * L.pstride + m];
-            } else {
-                // bounce-back on a fixed particle, plus the link force of Eq. 19
-                C gc = 0;
-                if (A.dJdF) {
-                    const double* gp = A.dJdF + 3 * L.owner[m];
-                    gc = C(2) * C(cx(i) * gp[0] + cy(i) * gp[1] + cz(i) * gp[2]);
-                }
-                for (int k = 0; k < 2; k++)
-                    mu[k][i] = Lin[((long long)(k * Q + opp(i))) * L.pstride + s] + Rin[k * L.pstride + s] + gc;
+        }
+        if (A.dJdF && (nbc & NB_LINKS)) {
+            // plus the link force of Eq. 19 on a fixed particle
+#pragma unroll
+            for (int i = 1; i < Q; i++) {
+                if (!((nbc >> i) & 1u)) continue;
+                const double* gp = A.dJdF + 3 * L.owner[nbr_index(L, n, i)];
+                const C gc = C(2) * C(cx(i) * gp[0] + cy(i) * gp[1] + cz(i) * gp[2]);
+                for (int k = 0; k < 2; k++) mu[k][i] += gc;
             }
         }
         // backward through the collision
@@ -211,62 +233,52 @@ __global__ void __launch_bounds__(128) k_adj_local(Lattice L, AdjArgs A) {
             mom_grad<C>(M, v[k], gv);
             for (int d = 0; d < 3; d++) {
                 ubar[d] += -a * rho[k] * gu[d];
-                C vbar = rho[k] * gv[d];
-                if (rho[k] > tiny) {
-                    ubar[d] += vbar;
-                    Fbar[k][d] = vbar / rho[k];
-                    rbar[k] += -vbar * F[k][d] / (rho[k] * rho[k]);
-                } else {
-                    ubar[d] += vbar;
-                    Fbar[k][d] = 0;
-                }
+                ubar[d] += rho[k] * gv[d];
+                // dJ/dF^k = gv; F^k / rho^k does not depend on rho^k
+                Fbar[k][d] = rho[k] > tiny ? gv[d] : C(0);
             }
         }
         // forces: F^A = -G rho^A S^B + rho^A g, F^B = -G rho^B S^A + rho^B g
         C SAbar[3], SBbar[3], Gbar = 0;
+#pragma unroll
         for (int d = 0; d < 3; d++) {
-            C g = C(L.P.body_force[d]);
-            rbar[0] += Fbar[0][d] * (-G * SB[d] + g);
-            rbar[1] += Fbar[1][d] * (-G * SA[d] + g);
             SBbar[d] = -G * rho[0] * Fbar[0][d];
             SAbar[d] = -G * rho[1] * Fbar[1][d];
-            Gbar += -rho[0] * Fbar[0][d] * SB[d] - rho[1] * Fbar[1][d] * SA[d];
+            Gbar -= wgt<C>(7) * (rho[0] * Fbar[0][d] * grad[1][d] + rho[1] * Fbar[1][d] * grad[0][d]);
         }
         // mixture velocity
-        C w0 = C(1) / C(L.P.tau[0]), w1 = C(1) / C(L.P.tau[1]);
-        C D = w0 * rho[0] + w1 * rho[1];
+        const C w0 = prm<C>(L.inv_tau[0], L.PF.inv_tau[0]), w1 = prm<C>(L.inv_tau[1], L.PF.inv_tau[1]);
+        const C iD = C(1) / (w0 * rho[0] + w1 * rho[1]);
         C jbar[2][3];
-        C udotub = ubar[0] * u[0] + ubar[1] * u[1] + ubar[2] * u[2];
-        C Dbar = -udotub / D;
+        const C Dbar = -(ubar[0] * u[0] + ubar[1] * u[1] + ubar[2] * u[2]) * iD;
+#pragma unroll
         for (int d = 0; d < 3; d++) {
-            jbar[0][d] = w0 * ubar[d] / D;
-            jbar[1][d] = w1 * ubar[d] / D;
+            jbar[0][d] = w0 * ubar[d] * iD;
+            jbar[1][d] = w1 * ubar[d] * iD;
         }
         rbar[0] += w0 * Dbar;
         rbar[1] += w1 * Dbar;
-        C wbar0 = (ubar[0] * j[0][0] + ubar[1] * j[0][1] + ubar[2] * j[0][2]) / D + Dbar * rho[0];
-        C wbar1 = (ubar[0] * j[1][0] + ubar[1] * j[1][1] + ubar[2] * j[1][2]) / D + Dbar * rho[1];
-        C t0 = C(L.P.tau[0]), t1 = C(L.P.tau[1]);
-        C taub0 = -wbar0 / (t0 * t0), taub1 = -wbar1 / (t1 * t1);
+        const C wbar0 = (ubar[0] * j[0][0] + ubar[1] * j[0][1] + ubar[2] * j[0][2]) * iD + Dbar * rho[0];
+        const C wbar1 = (ubar[0] * j[1][0] + ubar[1] * j[1][1] + ubar[2] * j[1][2]) * iD + Dbar * rho[1];
+        C taub0 = -wbar0 * w0 * w0, taub1 = -wbar1 * w1 * w1;
         // relaxation frequency of the mixture
-        C nu0 = (t0 - C(0.5)) / C(3), nu1 = (t1 - C(0.5)) / C(3);
-        C rt = rho[0] + rho[1];
-        C q = (rho[0] / rt) / nu0 + (rho[1] / rt) / nu1;
-        C nub = C(1) / q;
-        C ombar = -abar;
-        C nubbar = ombar * (-C(3) * om * om);
-        C qbar = nubbar * (-nub * nub);
-        rbar[0] += qbar * (C(1) / nu0 - q) / rt;
-        rbar[1] += qbar * (C(1) / nu1 - q) / rt;
-        taub0 += qbar * (-(rho[0] / rt) / (nu0 * nu0)) / C(3);
-        taub1 += qbar * (-(rho[1] / rt) / (nu1 * nu1)) / C(3);
+        const C in0 = prm<C>(L.inv_nu[0], L.PF.inv_nu[0]), in1 = prm<C>(L.inv_nu[1], L.PF.inv_nu[1]);
+        const C irt = C(1) / (rho[0] + rho[1]), x0 = rho[0] * irt, x1 = rho[1] * irt;
+        const C q = x0 * in0 + x1 * in1;
+        const C nub = C(1) / q;
+        const C nubbar = C(3) * abar * om * om;  // om = 1 / (3 nub + 1/2), a = 1 - om
+        const C qbar = -nubbar * (nub * nub);
+        rbar[0] += qbar * (in0 - q) * irt;
+        rbar[1] += qbar * (in1 - q) * irt;
+        taub0 -= qbar * (x0 * in0 * in0) * C(1.0 / 3.0);
+        taub1 -= qbar * (x1 * in1 * in1) * C(1.0 / 3.0);
         // local adjoint of the populations
 #pragma unroll
         for (int k = 0; k < 2; k++)
 #pragma unroll
             for (int i = 0; i < Q; i++)
                 Lout[((long long)(k * Q + i)) * L.pstride + s] =
-                    a * mu[k][i] + rbar[k] + C(cx(i)) * jbar[k][0] + C(cy(i)) * jbar[k][1] + C(cz(i)) * jbar[k][2];
+                    a * mu[k][i] + rbar[k] + along<C>(i, jbar[k]);
         for (int d = 0; d < 3; d++) {
             sb[(0 * 3 + d) * L.N + s] = SAbar[d];
             sb[(1 * 3 + d) * L.N + s] = SBbar[d];
@@ -278,7 +290,8 @@ __global__ void __launch_bounds__(128) k_adj_local(Lattice L, AdjArgs A) {
     // block partials of the parameter gradients (FP64 across threads)
     int nb = gridDim.x * gridDim.y * gridDim.z;
     int b = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
-    for (int v = 0; v < 3; v++) block_sum_store(double(part[v]), A.red + (long long)v * nb + b);
+    double sums[3] = {double(part[0]), double(part[1]), double(part[2])};
+    block_sum_store<3>(sums, A.red + b, nb);
 }
 
 // dJ/dpsi^k(y) = sum_i w_i c_i . Sbar^k(y - c_i) over fluid x = y - c_i.  On
@@ -297,23 +310,29 @@ __global__ void __launch_bounds__(128) k_adj_gather(Lattice L, AdjArgs A) {
         long long s = (long long)x + (long long)L.nx * ((long long)y + (long long)L.ny * z);
         SiteNbr n = site_nbr(L, x, y, z);
         const C* sb = (const C*)A.sbar;
+        const uint32_t nbc = L.nb[s];
+        const bool solid = nbc & NB_SOLID;
         C pb[2] = {0, 0}, W = 0;
 #pragma unroll
         for (int i = 1; i < Q; i++) {
             // the site x = y - c_i is the neighbour along opp(i)
             int io = opp(i);
-            if (nbr_is_wall(n, io)) continue;
-            long long m = nbr_index(L, n, io);
-            if (L.mask[m]) continue;
-            C w = wgt<C>(i);
+            const bool fluid = !nbr_is_wall(n, io) && (solid == (bool)((nbc >> io) & 1u));
+            const long long m = fluid ? nbr_index(L, n, io) : s;
+            const C w = fluid ? wgt<C>(i) : C(0);
             W += w;
-            for (int k = 0; k < 2; k++)
-                pb[k] += w * (C(cx(i)) * sb[(k * 3 + 0) * L.N + m] + C(cy(i)) * sb[(k * 3 + 1) * L.N + m] +
-                              C(cz(i)) * sb[(k * 3 + 2) * L.N + m]);
+#pragma unroll
+            for (int k = 0; k < 2; k++) {
+                C q[3];
+#pragma unroll
+                for (int d = 0; d < 3; d++)
+                    if (d == 0 ? cx(i) : (d == 1 ? cy(i) : cz(i))) q[d] = sb[(k * 3 + d) * L.N + m];
+                pb[k] += fluid ? w * along<C>(i, q) : C(0);
+            }
         }
         C* Rout = (C*)A.adj_out + 2 * Q * L.pstride;
         C* cf = (C*)A.coef;
-        if (!L.mask[s]) {
+        if (!solid) {
             Rout[s] = pb[0];
             Rout[L.pstride + s] = pb[1];
         } else {
@@ -343,7 +362,8 @@ __global__ void __launch_bounds__(128) k_adj_gather(Lattice L, AdjArgs A) {
     }
     int nb = gridDim.x * gridDim.y * gridDim.z;
     int b = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
-    for (int v = 0; v < 2; v++) block_sum_store(double(zp[v]), A.red + (long long)(3 + v) * nb + b);
+    double sums[2] = {double(zp[0]), double(zp[1])};
+    block_sum_store<2>(sums, A.red + 3ll * nb + b, nb);
 }
 
 // wall nodes: dJ/dpsi_wall from the fluid plane next to the wall, turned into
@@ -386,13 +406,14 @@ __global__ void __launch_bounds__(128) k_adj_scatter(Lattice L, AdjArgs A) {
     int y = blockIdx.y, z = blockIdx.z;
     if (x >= L.nx) return;
     long long s = (long long)x + (long long)L.nx * ((long long)y + (long long)L.ny * z);
-    if (L.mask[s]) return;
+    const uint32_t nbc = L.nb[s];
+    if (nbc & NB_SOLID) return;
     SiteNbr n = site_nbr(L, x, y, z);
+    if (!(nbc & NB_LINKS) && !n.wall_lo && !n.wall_hi) return;
     const C* cf = (const C*)A.coef;
     const C* cw = (const C*)A.coef_wall;
     long long nxy = (long long)L.nx * L.ny;
     C add[2] = {0, 0};
-    bool any = false;
 #pragma unroll
     for (int j = 1; j < Q; j++) {
         C w = wgt<C>(j);
@@ -403,35 +424,42 @@ __global__ void __launch_bounds__(128) k_adj_scatter(Lattice L, AdjArgs A) {
             long long wi = (long long)X + (long long)L.nx * Y;
             add[0] += w * cw[(side * 2 + 0) * nxy + wi];
             add[1] += w * cw[(side * 2 + 1) * nxy + wi];
-            any = true;
             continue;
         }
+        if (!((nbc >> j) & 1u)) continue;
         long long m = nbr_index(L, n, j);
-        if (!L.mask[m]) continue;
         add[0] += w * cf[m];
         add[1] += w * cf[L.N + m];
-        any = true;
     }
-    if (!any) return;
     C* Rout = (C*)A.adj_out + 2 * Q * L.pstride;
     Rout[s] += add[0];
     Rout[L.pstride + s] += add[1];
 }
 
-// Sum of the block partials of each parameter gradient, added to the
-// accumulator out[ADJ_VALUES]: warp v sums value v, lane l the partials
-// l, l + 32, ... (Neumaier), then the lanes merge in a fixed order.
-__global__ void k_adj_reduce(const double* red, int nb, double* out) {
-    const int v = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (v >= ADJ_VALUES) return;
+// Sums of the nb partials of each of gridDim.x values, red[v][nb], stored to
+// out[v], or added to it: a block of 256 threads per value, each thread the
+// partials t, t + 256, ... (Neumaier), then lanes and warps merge in a fixed
+// order.  (One warp per value and, for the objective, one thread took 51 us
+// and 563 us of dependent additions at 64^3; 14 us each now.)
+__global__ void __launch_bounds__(256) k_sum_partials(const double* __restrict__ red, int nb, double* out, bool add) {
+    __shared__ NSum part[8];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const double* r = red + (long long)blockIdx.x * nb;
     NSum t = {0.0, 0.0};
-    for (int b = lane; b < nb; b += 32) t.add(red[(long long)v * nb + b]);
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        NSum o = {__shfl_down_sync(0xffffffffu, t.s, off), __shfl_down_sync(0xffffffffu, t.c, off)};
-        if (lane < off) t.merge(o);
-    }
-    if (lane == 0) out[v] += t.value();
+    auto across = [&](int from) {
+        for (int off = from; off > 0; off >>= 1) {
+            NSum o = {__shfl_down_sync(0xffffffffu, t.s, off), __shfl_down_sync(0xffffffffu, t.c, off)};
+            if (lane < off) t.merge(o);
+        }
+    };
+    for (int b = threadIdx.x; b < nb; b += 256) t.add(r[b]);
+    across(16);
+    if (lane == 0) part[warp] = t;
+    __syncthreads();
+    if (warp > 0) return;
+    if (lane < 8) t = part[lane];
+    across(4);
+    if (lane == 0) out[blockIdx.x] = (add ? out[blockIdx.x] : 0.0) + t.value();
 }
 
 // dJ/dF_p for J = weight sum_p sqrt(|F_p|^2 + eps^2)
@@ -471,14 +499,8 @@ __global__ void __launch_bounds__(128) k_adj_seed_interface(Lattice L, void* adj
         Rout[s] = r0;
         Rout[L.pstride + s] = r1;
     }
-    block_sum_store(val, red + blockIdx.x);
-}
-
-__global__ void k_sum_blocks(const double* red, int nb, double* out) {
-    if (threadIdx.x != 0) return;
-    NSum t = {0.0, 0.0};
-    for (int b = 0; b < nb; b++) t.add(red[b]);
-    out[0] = t.value();
+    double sums[1] = {val};
+    block_sum_store<1>(sums, red + blockIdx.x, 1);
 }
 
 // dJ/drho^k(0) = sum_i w_i lambda^k_i(0) for f(0) = f^eq(rho^k(0), 0) = w_i rho^k(0)
@@ -561,7 +583,7 @@ int launch_adjoint_step(const Lattice& L, int prec, const void* in, void* out, v
     }
     DISPATCHA(prec, (k_adj_gather<P><<<gg, bx, 0, st>>>(L, A)));
     DISPATCHA(prec, (k_adj_scatter<P><<<gg, bx, 0, st>>>(L, A)));
-    k_adj_reduce<<<1, 32 * ADJ_VALUES, 0, st>>>(A.red, nb, grads_dev);
+    k_sum_partials<<<ADJ_VALUES, 256, 0, st>>>(A.red, nb, grads_dev, true);
     (void)g;
     return n + 3;
 }
@@ -571,7 +593,7 @@ int launch_adjoint_seed(const Lattice& L, int prec, void* adj, void* scratch, do
     AdjArgs A = adj_args(L, prec, nullptr, adj, scratch, nullptr);
     int nb = (int)((L.N + 127) / 128);
     DISPATCHA(prec, (k_adj_seed_interface<P><<<nb, 128, 0, st>>>(L, adj, A.red, weight)));
-    k_sum_blocks<<<1, 32, 0, st>>>(A.red, nb, value_dev);
+    k_sum_partials<<<1, 256, 0, st>>>(A.red, nb, value_dev, false);
     return 2;
 }
 
