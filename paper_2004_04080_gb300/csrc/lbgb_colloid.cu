@@ -78,16 +78,6 @@ __device__ __forceinline__ bool inside(const Lattice& L, int p, const PGeo<C>& g
     return inside_exact(L, p, a, b, c);
 }
 
-// |d| within [R + lo, R + hi) (in the compute type, with the margins chosen
-// by the callers well beyond its rounding): the shell where a kernel can have
-// work, so that the rest of the box is skipped without memory traffic
-template <typename C>
-__device__ __forceinline__ bool in_shell(const PGeo<C>& g, const C (&d)[3], float lo, float hi) {
-    float d2 = float(d[0]) * float(d[0]) + float(d[1]) * float(d[1]) + float(d[2]) * float(d[2]);
-    float a = float(g.R) + lo, b = float(g.R) + hi;
-    return (a <= 0.f || d2 >= a * a) && d2 < b * b;
-}
-
 // Visit the box points of particle p; f(X, Y, Z, s, a, b, c, d) gets the
 // wrapped site, its index, the unwrapped point and its offset from r_p.
 template <typename C, typename Fn>
@@ -111,43 +101,37 @@ __device__ __forceinline__ void for_box(const Lattice& L, const PGeo<C>& g, Fn&&
 }
 
 // Visit the box points of particle p whose distance from the centre lies in
-// [R + lo, R + hi) (the in_shell test, so the set is exactly that of a box
-// scan), one (y, z) row of the box per thread: the x range of a row that can
-// reach the shell is found from the row's distance to the centre (one or two
-// intervals, widened by a point on each side), so a thin shell costs its own
-// points instead of the whole box.  Sites are indexed in 32 bits.
+// [R + lo, R + hi), one (y, z) row of the box per thread: the x range of a row
+// that reaches the shell is found from the row's distance to the centre (one
+// or two intervals), so a thin shell costs its own points instead of the
+// whole box.  The shell is found in FP32 with a margin of 0.02 in x (far above
+// its rounding); what a point is, fn decides.  Sites are indexed in 32 bits.
 template <typename C, typename Fn>
 __device__ __forceinline__ void for_band(const Lattice& L, const PGeo<C>& g, float lo, float hi, Fn&& fn) {
+    constexpr float margin = 0.02f;
     const int tid = threadIdx.y * BXP + threadIdx.x;
     const int nrow = g.ext[1] * g.ext[2];
-    const float Rin = float(g.R) + lo, Rout = float(g.R) + hi;
-    const float cxr = float(g.ip[0]) + float(g.fr[0]);  // x of the centre (box frame)
+    const float Rin = fmaxf(float(g.R) + lo, 0.f), Rout = float(g.R) + hi;
+    const float fx = float(g.fr[0]), fy = float(g.fr[1]), fz = float(g.fr[2]);
     for (int r = tid; r < nrow; r += PB) {
-        const int b = g.lo[1] + r % g.ext[1], c = g.lo[2] + r / g.ext[1];
-        if (!L.per[2] && (c < 0 || c >= L.nz)) continue;
-        const C dy = C(b - g.ip[1]) - g.fr[1], dz = C(c - g.ip[2]) - g.fr[2];
-        const float q = float(dy) * float(dy) + float(dz) * float(dz);
-        const float ho = Rout * Rout - q;
-        if (ho < -1.f) continue;
-        const float xo = sqrtf(fmaxf(ho, 0.f)) + 1.f;
-        const float hin = Rin > 0.f ? Rin * Rin - q : -1.f;
-        const float xi = hin > 1.f ? sqrtf(hin) - 1.f : 0.f;  // |dx| >= xi can be in the shell
+        const int zz = r / g.ext[1], b = g.lo[1] + r - zz * g.ext[1], c = g.lo[2] + zz;
+        const float y = float(b - g.ip[1]) - fy, z = float(c - g.ip[2]) - fz;
+        const float q = y * y + z * z, ho = Rout * Rout - q, hin = Rin * Rin - q;
+        if (!(ho > 0.f) || (!L.per[2] && (c < 0 || c >= L.nz))) continue;
+        const float xo = sqrtf(ho) + margin, xi = hin > 0.f ? sqrtf(hin) - margin : 0.f;
         const int Y = b < 0 ? b + L.ny : (b >= L.ny ? b - L.ny : b);
         const int Z = c < 0 ? c + L.nz : (c >= L.nz ? c - L.nz : c);
         const int row = L.nx * (Y + L.ny * Z);
-        // x with |a - cx| in [xi, xo]: the left and right intervals (one if xi = 0)
-        const int aL0 = (int)floorf(cxr - xo), aL1 = (int)ceilf(cxr - xi);
-        const int aR0 = (int)floorf(cxr + xi), aR1 = (int)ceilf(cxr + xo);
-        const int split = xi > 0.f && aL1 < aR0;
-        for (int part = 0; part < 1 + split; part++) {
-            const int a0 = part == 0 ? aL0 : aR0, a1 = (part == 0 && split) ? aL1 : aR1;
-            for (int a = a0; a <= a1; a++) {
-                const C dx = C(a - g.ip[0]) - g.fr[0];
-                const C d[3] = {dx, dy, dz};
-                if (!in_shell<C>(g, d, lo, hi)) continue;
-                const int X = a < 0 ? a + L.nx : (a >= L.nx ? a - L.nx : a);
-                fn(X, Y, Z, (long long)(row + X), a, b, c, d);
-            }
+        // |x - r_p| in [xi, xo]: the left and right intervals (one if xi <= 0)
+        const int aL0 = (int)ceilf(fx - xo), aR1 = (int)floorf(fx + xo);
+        const int aL1 = xi > 0.f ? (int)floorf(fx - xi) : aR1, aR0 = xi > 0.f ? (int)ceilf(fx + xi) : aR1 + 1;
+        const int nl = aL1 - aL0 + 1, total = max(nl, 0) + max(aR1 - aR0 + 1, 0);
+        for (int t = 0; t < total; t++) {
+            const int a = t < nl ? aL0 + t : aR0 + t - max(nl, 0);
+            const int ax = a + g.ip[0];
+            const C d[3] = {C(a) - g.fr[0], C(b - g.ip[1]) - g.fr[1], C(c - g.ip[2]) - g.fr[2]};
+            const int X = ax < 0 ? ax + L.nx : (ax >= L.nx ? ax - L.nx : ax);
+            fn(X, Y, Z, (long long)(row + X), ax, b, c, d);
         }
     }
 }
@@ -272,7 +256,8 @@ __device__ __forceinline__ void particle_frame(const Lattice& L, int p, int x, i
 // the 0.65, so that particles which overlapped before it are reported by every
 // call that steps them.  A shell of 0.65 for every particle read the
 // owner map of ten times the points: 512 x 512 x 256, 14,444 particles, 302
-// us against 105.
+// us against 101 (96^3 FP64: 90 against 27).  Points outside the shell are found
+// in FP32 before any FP64 distance is formed (39 us before at 96^3).
 template <int PREC, bool MOM>
 __global__ void __launch_bounds__(PB) k_remap_classify(const __grid_constant__ Lattice L, bool wide) {
     typedef typename Prec<PREC>::C C;
@@ -858,87 +843,72 @@ __global__ void __launch_bounds__(128) k_pairs(Lattice L) {
 // form qdot = ((0, w) q / 2 - w.w q / 8) / (1 + w.w / 16), the fixed point of
 // the iteration that Eq. 34 prescribes.  (Iterated, with two roots and eight
 // divisions in FP64 each time: 40 us a step whatever the number of particles,
-// FP64 running two lanes a cycle on an SM; 11 us now, in blocks of one warp.)
+// FP64 running two lanes a cycle on an SM; one thread per particle took 11 us,
+// four lanes, one per axis and component of the quaternion, take 8.6 us with 801
+// particles, and 14.7 instead of 23 with 14,444.)
 __global__ void __launch_bounds__(32) k_integrate(const __grid_constant__ Lattice L) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p == 0) *L.nb_chg = 0;
-    if (p >= L.nc) return;
-    double t[ACC_TERMS][3], Fp[3], Tp[3], pair[3], r[3], v[3], w[3], q[4];
+    const int t = blockIdx.x * blockDim.x + threadIdx.x, d = t & 3, a = d < 3 ? d : 0, p = min(t >> 2, L.nc - 1);
+    const bool live = (t >> 2) < L.nc, axis = live && d < 3;
+    const unsigned all = 0xffffffffu;
+    if (t == 0) *L.nb_chg = 0;
+    const int i = 3 * p + a;
+    double term[ACC_TERMS];
 #pragma unroll
-    for (int a = 0; a < ACC_TERMS; a++)
-#pragma unroll
-        for (int d = 0; d < 3; d++) {
-            unsigned long long* slot = acc_slot(L, a, p, d);
-            t[a][d] = acc_value(L, slot);
-            slot[0] = slot[1] = 0ull;
-        }
+    for (int k = 0; k < ACC_TERMS; k++) term[k] = acc_value(L, acc_slot(L, k, p, a));
     const bool first = !L.prev_valid[p];
-#pragma unroll
-    for (int d = 0; d < 3; d++) {
-        Fp[d] = L.Fliq_prev[3 * p + d];
-        Tp[d] = L.Tliq_prev[3 * p + d];
-        pair[d] = L.Fpair[3 * p + d];
-        r[d] = L.pos[3 * p + d];
-        v[d] = L.vel[3 * p + d];
-        w[d] = L.omg[3 * p + d];
-    }
-#pragma unroll
-    for (int d = 0; d < 4; d++) q[d] = L.quat[4 * p + d];
+    const double Fp = first ? term[ACC_FLIQ] : L.Fliq_prev[i], Tp = first ? term[ACC_TLIQ] : L.Tliq_prev[i];
     const double im = 1.0 / L.mass[p], R = L.rad[p];
-    double* terms[ACC_TERMS] = {L.Fliq, L.Tliq, L.Fd, L.Td, L.Fc, L.Tc, L.Fs, L.Ts};
+    double v = L.vel[i], r = L.pos[i], w = L.omg[i], q = L.quat[4 * p + d];
+    const double F = 0.5 * (Fp + term[ACC_FLIQ]) + term[ACC_FD] + term[ACC_FC] + term[ACC_FS] + L.Fpair[i];
+    const double T = 0.5 * (Tp + term[ACC_TLIQ]) + term[ACC_TD] + term[ACC_TC] + term[ACC_TS];
+    const int n = a == 0 ? L.nx : (a == 1 ? L.ny : L.nz);
+    v += F * im;
+    r += v;
+    if (L.per[a] && !(r >= 0.0 && r < (double)n)) r = r - (double)n * floor(r / (double)n);
+    __syncwarp(all);  // every lane has read the sums and prev_valid
+    if (axis) {
+        double* terms[ACC_TERMS] = {L.Fliq, L.Tliq, L.Fd, L.Td, L.Fc, L.Tc, L.Fs, L.Ts};
 #pragma unroll
-    for (int a = 0; a < ACC_TERMS; a++)
-#pragma unroll
-        for (int d = 0; d < 3; d++) terms[a][3 * p + d] = t[a][d];
-    const int Ls[3] = {L.nx, L.ny, L.nz};
-    bool fast = false;
-    double T[3];
-#pragma unroll
-    for (int d = 0; d < 3; d++) {
-        const double fp = first ? t[ACC_FLIQ][d] : Fp[d], tp = first ? t[ACC_TLIQ][d] : Tp[d];
-        const double F = 0.5 * (fp + t[ACC_FLIQ][d]) + t[ACC_FD][d] + t[ACC_FC][d] + t[ACC_FS][d] + pair[d];
-        T[d] = 0.5 * (tp + t[ACC_TLIQ][d]) + t[ACC_TD][d] + t[ACC_TC][d] + t[ACC_TS][d];
-        L.Ftot[3 * p + d] = F;
-        L.Ttot[3 * p + d] = T[d];
-        L.Fliq_prev[3 * p + d] = t[ACC_FLIQ][d];
-        L.Tliq_prev[3 * p + d] = t[ACC_TLIQ][d];
-        v[d] += F * im;
-        r[d] += v[d];
-        if (L.per[d] && !(r[d] >= 0.0 && r[d] < (double)Ls[d])) r[d] = r[d] - double(Ls[d]) * floor(r[d] / double(Ls[d]));
-        fast |= !(fabs(v[d]) < 0.5);
-        L.vel[3 * p + d] = v[d];
-        L.pos[3 * p + d] = r[d];
+        for (int k = 0; k < ACC_TERMS; k++) {
+            unsigned long long* slot = acc_slot(L, k, p, a);
+            slot[0] = slot[1] = 0ull;
+            terms[k][i] = term[k];
+        }
+        L.Ftot[i] = F;
+        L.Ttot[i] = T;
+        L.Fliq_prev[i] = term[ACC_FLIQ];
+        L.Tliq_prev[i] = term[ACC_TLIQ];
+        L.vel[i] = v;
+        L.pos[i] = r;
+        if (!(fabs(v) < 0.5)) atomicOr(L.flags, FLAG_NONFINITE);
+        if (a == 0) L.prev_valid[p] = 1;
     }
-    if (fast) atomicOr(L.flags, FLAG_NONFINITE);
-    L.prev_valid[p] = 1;
     if (L.P.rotate) {
-        const double iI = im / (0.4 * R * R);
-        double ww = 0.0, nq = 0.0;
-#pragma unroll
-        for (int d = 0; d < 3; d++) {
-            w[d] += T[d] * iI;
-            ww += w[d] * w[d];
-            L.omg[3 * p + d] = w[d];
-        }
-        const double s = 1.0 / (1.0 + 0.0625 * ww);
-        const double wq[4] = {-(w[0] * q[1] + w[1] * q[2] + w[2] * q[3]), w[0] * q[0] + w[1] * q[3] - w[2] * q[2],
-                              w[1] * q[0] + w[2] * q[1] - w[0] * q[3], w[2] * q[0] + w[0] * q[2] - w[1] * q[1]};
-#pragma unroll
-        for (int d = 0; d < 4; d++) {
-            q[d] += (0.5 * wq[d] - 0.125 * ww * q[d]) * s;
-            nq += q[d] * q[d];
-        }
-        const double in = 1.0 / sqrt(nq);
-#pragma unroll
-        for (int d = 0; d < 4; d++) L.quat[4 * p + d] = q[d] * in;
+        w += T * (im / (0.4 * R * R));
+        const double w0 = __shfl_sync(all, w, 0, 4), w1 = __shfl_sync(all, w, 1, 4), w2 = __shfl_sync(all, w, 2, 4);
+        const double q0 = __shfl_sync(all, q, 0, 4), q1 = __shfl_sync(all, q, 1, 4), q2 = __shfl_sync(all, q, 2, 4),
+                     q3 = __shfl_sync(all, q, 3, 4);
+        const double ww = w0 * w0 + w1 * w1 + w2 * w2;
+        // component d of (0, w) q
+        const double x = d == 0 ? -w0 : (d == 1 ? w0 : (d == 2 ? w1 : w2));
+        const double y = d == 0 ? -w1 : (d == 1 ? w1 : (d == 2 ? w2 : w0));
+        const double z = d == 0 ? -w2 : (d == 1 ? -w2 : (d == 2 ? -w0 : -w1));
+        const double wq = x * (d == 0 ? q1 : q0) + y * (d == 1 ? q3 : (d == 2 ? q1 : q2)) +
+                          z * (d == 0 || d == 2 ? q3 : (d == 1 ? q2 : q1));
+        q += (0.5 * wq - 0.125 * ww * q) / (1.0 + 0.0625 * ww);
+        double nq = q * q;
+        nq += __shfl_xor_sync(all, nq, 1, 4);
+        nq += __shfl_xor_sync(all, nq, 2, 4);
+        q = q / sqrt(nq);
+        if (axis) L.omg[i] = w;
+        if (live) L.quat[4 * p + d] = q;
     }
-#pragma unroll
-    for (int d = 0; d < 3; d++) {
-        const int ip = (int)floor(r[d]);
-        L.ipos[3 * p + d] = ip;
-        L.fsnap[9 * p + d] = float(r[d] - (double)ip);
-        L.fsnap[9 * p + 3 + d] = float(v[d]);
-        L.fsnap[9 * p + 6 + d] = float(w[d]);
+    if (axis) {
+        const int ip = (int)floor(r);
+        L.ipos[i] = ip;
+        L.fsnap[9 * p + a] = float(r - (double)ip);
+        L.fsnap[9 * p + 3 + a] = float(v);
+        L.fsnap[9 * p + 6 + a] = float(w);
     }
 }
 
@@ -1056,7 +1026,7 @@ int launch_pairs(const Lattice& L, void* cells, size_t cell_cap, bool force_buil
 
 int launch_integrate(const Lattice& L, cudaStream_t st) {
     if (L.nc <= 0) return 0;
-    k_integrate<<<(L.nc + 31) / 32, 32, 0, st>>>(L);
+    k_integrate<<<(L.nc + 7) / 8, 32, 0, st>>>(L);
     return 1;
 }
 
