@@ -62,6 +62,16 @@ def kernel_bytes(kname, prec):
     return 2 * pops + 1
 
 
+def run_bytes(kname, prec, steps):
+    """(lattice kernel, bytes per site) of the steps of a call of ``steps``
+    steps whose last one runs ``kname``: at tau = 1 in FP32 and FP16 the others
+    go from moments to moments (rho of one component and j, or rho^k and j, read
+    and written); else a step reads and writes the populations."""
+    if steps > 1 and prec != "fp64" and kname in ("k_lean", "k1_step"):
+        return "k_moments", kernel_bytes("k_moments", prec) if kname == "k_lean" else 8 * COMPUTE[prec]
+    return kname, alg_bytes(prec) if kname != "k1_step" else 38 * STORE[prec]
+
+
 DTYPE = {"fp64": "f64", "fp32": "f32", "fp16": "f16-storage/f32-math"}
 # stated parity bounds against the FP64 oracle (relative, fields after 100 steps), as tested
 STATED_ERROR = {"fp64": 1e-12, "fp32": 1e-5, "fp16": 1e-3}
@@ -353,11 +363,12 @@ def case0_throughput(dev, torch, n=1024, steps=10):
     del rhoA, rhoB
     lat.step(2)
     ms = time_steps(lat, steps, torch)
+    kname, nbytes = run_bytes(lat.fused_kernel(), "fp16", steps)
     out = {"workload": "%d^3 periodic, two components, G = 0.65, rho = 1.0 + 1.0 (std 0.004), tau = 1, "
                        "no particles, FP16 storage (stochastic rounding)" % n,
            "steps": steps, "ms_per_step": round(ms / steps, 3), "glups": round(N * steps / (ms / 1e3) / 1e9, 3),
-           "kernel": lat.fused_kernel(), "bytes_per_site": alg_bytes("fp16"),
-           "hbm_frac": round(N * steps / (ms / 1e3) * alg_bytes("fp16") / 1e9 / peaks()[0], 4),
+           "kernel": kname, "bytes_per_site": nbytes,
+           "hbm_frac": round(N * steps / (ms / 1e3) * nbytes / 1e9 / peaks()[0], 4),
            "paper_glups": 1.37, "paper_case": "1024^3 case 0 on 1024 cores (Sec. 5.1 two-component table)"}
     del lat
     torch.cuda.empty_cache()
@@ -385,10 +396,11 @@ def single_throughput(dev, torch, n=1024, steps=10):
     del rho
     lat.step(2)
     ms = time_steps(lat, steps, torch)
+    kname, nbytes = run_bytes(lat.fused_kernel(), "fp32", steps)
     out = {"workload": "%d^3 periodic, one component, rho = 1.0 (Gaussian, std 1e-4), tau = 1, FP32 storage" % n,
            "steps": steps, "ms_per_step": round(ms / steps, 3), "glups": round(N * steps / (ms / 1e3) / 1e9, 3),
-           "kernel": lat.fused_kernel(), "bytes_per_site": 152,
-           "hbm_frac": round(152 * N * steps / (ms / 1e3) / 1e9 / peaks()[0], 4),
+           "kernel": kname, "bytes_per_site": nbytes,
+           "hbm_frac": round(nbytes * N * steps / (ms / 1e3) / 1e9 / peaks()[0], 4),
            "paper_glups": 6.51, "paper_case": "1024^3 single component on 2048 cores (Sec. 5.1 first table)"}
     del lat
     torch.cuda.empty_cache()
@@ -467,8 +479,7 @@ def main():
     value, ms = replica_mlups(ms, w.n_sites, args.steps, world, dev)
     ms_step = ms / args.steps
     peak, peak_kind = peaks()
-    kname = lat.fused_kernel()
-    abytes = alg_bytes(args.prec)
+    steps_kname, abytes = run_bytes(lat.fused_kernel(), args.prec, args.steps)
     alg = abytes * w.n_sites
     # per step: at tau = 1 the steps of a call between the first and the last
     # run from moments to moments, and the density pass runs once a call
@@ -476,13 +487,10 @@ def main():
     davg = dens_ms / max(kern_n, 1)
     traffic = recorded_traffic(args.prec)
     # frac is the rate of the lattice kernels against the measured copy
-    # bandwidth for one read and one write of every population a step (the
-    # bytes of a step that keeps its state in populations: above 1 where the
-    # steps of a call keep rho^k and j instead, whose own bytes are in
-    # `kernels`); step_frac the same bytes over the whole step.
+    # bandwidth for the bytes such a step has to move (its state read and
+    # written once); step_frac the same bytes over the whole step.
     lattice_ms = kavg + davg
     achieved = alg / (lattice_ms / 1e3) / 1e9
-    steps_kname = "k_moments" if dens_n < kern_n and kname == "k_lean" else kname
     kernels = [{"kernel": steps_kname, "ms": round(kavg, 4), "own_bytes_per_site": kernel_bytes(steps_kname, args.prec),
                 "own_frac": round(kernel_bytes(steps_kname, args.prec) * w.n_sites / (kavg / 1e3) / 1e9 / peak, 4)}]
     if dens_n == kern_n:
@@ -549,9 +557,10 @@ def main():
             km, kn = L2.profile_read()
             dm, dn = L2.profile_read(LB_KERNEL_DENSITY)
             kk = (km + dm) / max(kn, 1)
+            fk, fbytes = run_bytes(L2.fused_kernel(), prec, steps)
             forms[prec] = {"mlups": round(world * N * steps / (m2 / 1e3) / 1e6, 1), "steps": steps,
-                           "kernel": L2.fused_kernel(),
-                           "kernel_frac": round(alg_bytes(prec) * N / (kk / 1e3) / 1e9 / peak, 4),
+                           "kernel": fk, "bytes_per_site": fbytes,
+                           "kernel_frac": round(fbytes * N / (kk / 1e3) / 1e9 / peak, 4),
                            "stated_rel_error_vs_fp64_oracle": STATED_ERROR[prec]}
             if prec == "fp16":
                 forms[prec]["rounding"] = "stochastic (cvt.rs.f16x2.f32, the FP16 default)"
