@@ -260,6 +260,7 @@ __device__ __forceinline__ void particle_frame(const Lattice& L, int p, int x, i
 // in FP32 before any FP64 distance is formed (39 us before at 96^3).
 template <int PREC, bool MOM>
 __global__ void __launch_bounds__(PB) k_remap_classify(const __grid_constant__ Lattice L, bool wide) {
+    chain_begin();
     typedef typename Prec<PREC>::C C;
     int p = blockIdx.x;
     PGeo<C> g = pgeo<C>(L, p, REMAP_PAD);
@@ -363,6 +364,7 @@ __device__ __forceinline__ void refill_node(const Lattice& L, long long s, int p
 // other, 39 us a step at 128^3 with 801 particles against 6.
 template <int PREC, bool MOM>
 __global__ void __launch_bounds__(128) k_remap_create(const __grid_constant__ Lattice L) {
+    chain_begin();
     const int cnt = *L.nb_chg, lane = threadIdx.x & 31;
     const int warp = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), nw = (int)(gridDim.x * blockDim.x >> 5);
     if (cnt <= NB_CHG_CAP) {
@@ -385,6 +387,7 @@ __global__ void __launch_bounds__(128) k_remap_create(const __grid_constant__ La
 // Commit the new node map.
 template <int PREC, bool MOM>
 __global__ void k_remap_commit(const __grid_constant__ Lattice L) {
+    chain_begin();
     const int cnt = *L.nb_chg;
     const bool listed = cnt <= NB_CHG_CAP;
     const long long n = listed ? cnt : L.N;
@@ -441,6 +444,7 @@ __global__ void k_link_classes_all(Lattice L) {
 // final): a site next to two changed nodes is rewritten with the same word
 // by both.  When more nodes changed than the list holds, every site.
 __global__ void k_link_classes_changed(Lattice L) {
+    chain_begin();
     const int cnt = *L.nb_chg;
     const long long nt = (long long)gridDim.x * blockDim.x;
     long long t0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -491,6 +495,7 @@ constexpr int VTX = 32, VTY = 8, VZC = 16;  // tile and planes per block (4096 s
 
 template <int PREC>
 __global__ void __launch_bounds__(VTX* VTY) k_virtual(const __grid_constant__ Lattice L, int store_terms, int zc) {
+    chain_begin();
     typedef typename Prec<PREC>::C C;
     struct alignas(2 * sizeof(C)) Pair {
         C a, b;
@@ -847,6 +852,7 @@ __global__ void __launch_bounds__(128) k_pairs(Lattice L) {
 // four lanes, one per axis and component of the quaternion, take 8.6 us with 801
 // particles, and 14.7 instead of 23 with 14,444.)
 __global__ void __launch_bounds__(32) k_integrate(const __grid_constant__ Lattice L) {
+    chain_begin();
     const int t = blockIdx.x * blockDim.x + threadIdx.x, d = t & 3, a = d < 3 ? d : 0, p = min(t >> 2, L.nc - 1);
     const bool live = (t >> 2) < L.nc, axis = live && d < 3;
     const unsigned all = 0xffffffffu;
@@ -937,8 +943,8 @@ int launch_map_initial(const Lattice& L, int prec, int first, int count, cudaStr
 template <int P, bool MOM>
 static void launch_remap_t(const Lattice& L, bool wide, cudaStream_t st) {
     k_remap_classify<P, MOM><<<L.nc, PBLK, 0, st>>>(L, wide);
-    k_remap_create<P, MOM><<<(unsigned)(16 * device_sms()), 128, 0, st>>>(L);
-    k_remap_commit<P, MOM><<<(unsigned)(2 * device_sms()), 128, 0, st>>>(L);
+    launch_after(k_remap_create<P, MOM>, (unsigned)(16 * device_sms()), 128, 0, st, L);
+    launch_after(k_remap_commit<P, MOM>, (unsigned)(2 * device_sms()), 128, 0, st, L);
 }
 
 int launch_clear_terms(const Lattice& L, cudaStream_t st) {
@@ -963,7 +969,7 @@ int launch_link_classes(const Lattice& L, bool full, cudaStream_t st) {
         const int bx = L.nx >= 128 ? 128 : ((L.nx + 31) / 32) * 32;
         k_link_classes_all<<<dim3((unsigned)((L.nx + bx - 1) / bx), (unsigned)L.ny, (unsigned)L.nz), bx, 0, st>>>(L);
     } else {
-        k_link_classes_changed<<<(unsigned)(4 * device_sms()), 256, 0, st>>>(L);
+        launch_after(k_link_classes_changed, (unsigned)(4 * device_sms()), 256, 0, st, L);
     }
     return 1;
 }
@@ -976,7 +982,7 @@ int launch_virtual(const Lattice& L, int prec, int store_terms, cudaStream_t st)
     const long long zw = tiles * L.nz / (4 * device_sms());
     const int zc = (int)(zw < 2 ? 2 : (zw > VZC ? VZC : zw));
     dim3 grid((L.nx + VTX - 1) / VTX, (L.ny + VTY - 1) / VTY, (L.nz + zc - 1) / zc);
-    DISPATCHC(prec, (k_virtual<P><<<grid, dim3(VTX, VTY), 0, st>>>(L, store_terms, zc)));
+    DISPATCHC(prec, (launch_after(k_virtual<P>, grid, dim3(VTX, VTY), 0, st, L, store_terms, zc)));
     return 1;
 }
 

@@ -686,6 +686,35 @@ __device__ __forceinline__ void cp_async_8(void* dst, const void* src) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
+// ------------------------------------------------ kernels of a step in a row
+// A step is a chain of kernels of a few us each on a small lattice.  A kernel
+// launched by launch_after may be set up, and its blocks placed, while the
+// one before it on the stream still runs: chain_begin, the first statement of
+// every such kernel, lets the next one do the same and then waits until the
+// one before has ended and its writes are seen (each kernel of the chain waits
+// for its predecessor before it ends, so all earlier ones have ended too).
+// A call of one step at 32^3 FP32 83 -> 66 us, a step at 128^3 161 -> 149, at
+// 140x92x110 with unequal tau 255 -> 242, one adjoint gradient at 64^3 12.1 -> 10.8 ms.
+__device__ __forceinline__ void chain_begin() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+template <typename... P, typename... A>
+static void launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t c = {};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    cudaLaunchKernelEx(&c, kernel, P(args)...);
+}
+
 // ------------------------------------------------ per-device launch state
 // The > 48 KB dynamic shared-memory attribute is a property of a function in
 // one CUDA context, and the resident-block and SM counts that size the grids

@@ -395,6 +395,7 @@ template <int NK, bool PART>
 __global__ void __launch_bounds__(MNT, NK == 1 ? 4 : 3)
     k_moments(const __grid_constant__ Lattice L, float* __restrict__ psi_o, float* __restrict__ mom_o, LinkList list,
               int zc, int TW) {
+    chain_begin();
     typedef MomentShared<NK, PART> SH;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SH& sh = *reinterpret_cast<SH*>(smem_raw);
@@ -706,6 +707,7 @@ __global__ void __launch_bounds__(MNT, NK == 1 ? 4 : 3)
 __global__ void __launch_bounds__(128) k_bounce_links(const __grid_constant__ Lattice L, float* __restrict__ psi_o,
                                                        float* __restrict__ mom_o, LinkList list, int zc, int TW,
                                                        int parts, long long unit) {
+    chain_begin();
     const int bx = blockIdx.x / parts, z0 = blockIdx.z * zc, x0 = bx * TW, y0 = blockIdx.y * MROWS;
     const int n = list.count[bx + gridDim.x / parts * (blockIdx.y + gridDim.y * blockIdx.z)];
     const unsigned* seg = list.rec + segment_of(L, x0, y0, min(MROWS, L.ny - y0), z0, min(zc, L.nz - z0));
@@ -851,6 +853,7 @@ __global__ void __launch_bounds__(128) k_bounce_links(const __grid_constant__ La
 // links into the face from psi and mom of time t.
 template <int NK>
 __global__ void k_moment_faces(const __grid_constant__ Lattice L, float* __restrict__ psi_o, float* __restrict__ mom_o) {
+    chain_begin();
     const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y, face = blockIdx.z;
     if (x >= L.nx) return;
     const int z = face == 0 ? 0 : L.nz - 1;
@@ -955,7 +958,7 @@ static int launch_moments_t(const Lattice& L, void* psi_o, void* mom_o, cudaStre
     LinkList list = {(unsigned*)L.f_nxt, (int*)L.f_nxt + (size_t)MREC * L.N};
     float *po = (float*)psi_o, *mo = (float*)mom_o;
     int n = 1;
-    k_moments<NK, PART><<<grid, MNT, smem, st>>>(L, po, mo, list, zc, TW);
+    launch_after(k_moments<NK, PART>, grid, MNT, smem, st, L, po, mo, list, zc, TW);
     if (PART) {
         // about a fifth of the sites are boundary sites in a dense suspension:
         // blocks for two or three rounds over a segment
@@ -963,7 +966,7 @@ static int launch_moments_t(const Lattice& L, void* psi_o, void* mom_o, cudaStre
         // what a link of weight 1/36 of the reference fluid hands over (2 f*_i of
         // both components), in fixed point
         const long long unit = llrint(((double)L.rref[0] + (double)L.rref[1]) * (2.0 / 36.0 * 1099511627776.0));
-        k_bounce_links<<<dim3(gx * parts, gy, grid.z), 128, 0, st>>>(L, po, mo, list, zc, TW, parts, unit);
+        launch_after(k_bounce_links, dim3(gx * parts, gy, grid.z), 128, 0, st, L, po, mo, list, zc, TW, parts, unit);
         n++;
     }
     if (!L.per[2]) {
