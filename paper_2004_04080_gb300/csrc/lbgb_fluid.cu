@@ -57,17 +57,27 @@ __global__ void k_density(Lattice L) {
         return;
     }
     const S* f = (const S*)L.f_cur;
-    // j from the differences of opposite links of both components (39
-    // additions; 60 link by link: 96^3 in FP64, which the additions bound, 182
-    // -> 147 us for the whole pass)
-    C rho[2] = {0, 0}, jt[3] = {0, 0, 0}, last[2] = {0, 0};
+    // FP64: j from the differences of opposite links of both components (39
+    // additions, 60 link by link: 96^3, which the additions bound, 182 -> 147 us
+    // for the whole pass).  FP32 and FP16 are bound by memory and sum link by
+    // link: the last bits of a recorded run then stay those of earlier versions,
+    // and with them gradients through it (36 steps at 64^3: the parameters'
+    // gradients 1.0e-6 from their values in 64 bits at most, 1.3e-6 by pairs).
+    C rho[2] = {0, 0}, jt[3] = {0, 0, 0}, jk[2][3] = {{0, 0, 0}, {0, 0, 0}}, last[2] = {0, 0};
 #pragma unroll
     for (int i = 0; i < Q; i++) {
         C v[2];
         ld_pair(f + pair_index(i, s, L.pstride), pop_shift<S, C>(L, 0, i), pop_shift<S, C>(L, 1, i), v[0], v[1]);
 #pragma unroll
         for (int k = 0; k < 2; k++) rho[k] += v[k];
-        if (MOM && i > 0 && i == opp(i - 1)) {
+        if (MOM && PREC != LB_FP64)
+#pragma unroll
+            for (int k = 0; k < 2; k++) {
+                if (cx(i) > 0) jk[k][0] += v[k]; else if (cx(i) < 0) jk[k][0] -= v[k];
+                if (cy(i) > 0) jk[k][1] += v[k]; else if (cy(i) < 0) jk[k][1] -= v[k];
+                if (cz(i) > 0) jk[k][2] += v[k]; else if (cz(i) < 0) jk[k][2] -= v[k];
+            }
+        if (MOM && PREC == LB_FP64 && i > 0 && i == opp(i - 1)) {
             const C d = (last[0] - v[0]) + (last[1] - v[1]);  // along c_(i - 1)
             if (cx(i) < 0) jt[0] += d; else if (cx(i) > 0) jt[0] -= d;
             if (cy(i) < 0) jt[1] += d; else if (cy(i) > 0) jt[1] -= d;
@@ -76,6 +86,9 @@ __global__ void k_density(Lattice L) {
         last[0] = v[0];
         last[1] = v[1];
     }
+    if (MOM && PREC != LB_FP64)
+#pragma unroll
+        for (int d = 0; d < 3; d++) jt[d] = jk[0][d] + jk[1][d];
     psi[2 * s] = rho[0];
     psi[2 * s + 1] = rho[1];
     if (MOM)
@@ -904,22 +917,59 @@ __device__ __forceinline__ void lean_site(const Lattice& L, const LeanShared<PRE
     C rho[2];
 #pragma unroll
     for (int k = 0; k < 2; k++) rho[k] = solid ? prm<C>(L.P.rho0[k], L.PF.rho0[k]) : sh.psi[sl[1]][1][tx + 1][k];
-    // Eq. 11 (repulsive sign) + body force from the staged psi planes, per
-    // density: F^k / rho^k = g - G S
-    C grad[2][3];
-    link_gradient<C>(grad, [&](int i, int k) { return sh.psi[sl[cz(i) + 1]][1 + cy(i)][tx + 1 + cx(i)][k]; });
-    const C G36 = prm<C>(L.P.G, L.PF.G) * wgt<C>(7);
-    // Eq. 14 at tau_A = tau_B: u = (j^A + j^B) / (rho^A + rho^B) (j = 0 on
-    // particle nodes); Eq. 16: the shifted velocities
     C us[2][3];
-    {
-        const C ir = C(1) / (rho[0] + rho[1]);
+    // FP64, which the operations bound: by opposite pairs and without divisions.
+    // FP32 and FP16 sum link by link (see k_density: the same last bits)
+    if constexpr (PREC == LB_FP64) {
+        // Eq. 11 (repulsive sign) + body force from the staged psi planes, per
+        // density: F^k / rho^k = g - G S
+        C grad[2][3];
+        link_gradient<C>(grad, [&](int i, int k) { return sh.psi[sl[cz(i) + 1]][1 + cy(i)][tx + 1 + cx(i)][k]; });
+        const C G36 = prm<C>(L.P.G, L.PF.G) * wgt<C>(7);
+        // Eq. 14 at tau_A = tau_B: u = (j^A + j^B) / (rho^A + rho^B) (j = 0 on
+        // particle nodes); Eq. 16: the shifted velocities
+        {
+            const C ir = C(1) / (rho[0] + rho[1]);
+            const C tiny = sizeof(C) == 8 ? C(1e-300) : C(1e-30);
+#pragma unroll
+            for (int d = 0; d < 3; d++) {
+                const C u = sh.j[b][d][tx] * ir, g = prm<C>(L.P.body_force[d], L.PF.body_force[d]);
+#pragma unroll
+                for (int k = 0; k < 2; k++) us[k][d] = u + (rho[k] > tiny ? g - G36 * grad[1 - k][d] : C(0));
+            }
+        }
+    } else {
+        // Eq. 11 (repulsive sign) + body force from the staged psi planes
+        C sA[3] = {0, 0, 0}, sB[3] = {0, 0, 0};
+#pragma unroll
+        for (int i = 1; i < Q; i++) {
+            const int slot = sl[cz(i) + 1];
+            const C pa = sh.psi[slot][1 + cy(i)][tx + 1 + cx(i)][0];
+            const C pb = sh.psi[slot][1 + cy(i)][tx + 1 + cx(i)][1];
+            const C w = wgt<C>(i);
+            if (cx(i)) { sA[0] += C(cx(i)) * w * pa; sB[0] += C(cx(i)) * w * pb; }
+            if (cy(i)) { sA[1] += C(cy(i)) * w * pa; sB[1] += C(cy(i)) * w * pb; }
+            if (cz(i)) { sA[2] += C(cz(i)) * w * pa; sB[2] += C(cz(i)) * w * pb; }
+        }
+        const C G = prm<C>(L.P.G, L.PF.G);
+        // Eq. 14 at tau_A = tau_B: u = (j^A + j^B) / (rho^A + rho^B) (j = 0 on
+        // particle nodes)
+        C u[3];
+        {
+            const C ir = C(1) / (rho[0] + rho[1]);
+#pragma unroll
+            for (int d = 0; d < 3; d++) u[d] = sh.j[b][d][tx] * ir;
+        }
         const C tiny = sizeof(C) == 8 ? C(1e-300) : C(1e-30);
 #pragma unroll
-        for (int d = 0; d < 3; d++) {
-            const C u = sh.j[b][d][tx] * ir, g = prm<C>(L.P.body_force[d], L.PF.body_force[d]);
+        for (int k = 0; k < 2; k++) {
+            const C ir = rho[k] > tiny ? C(1) / rho[k] : C(0);
 #pragma unroll
-            for (int k = 0; k < 2; k++) us[k][d] = u + (rho[k] > tiny ? g - G36 * grad[1 - k][d] : C(0));
+            for (int d = 0; d < 3; d++) {
+                const C g = prm<C>(L.P.body_force[d], L.PF.body_force[d]);
+                const C F = -G * rho[k] * (k == 0 ? sB[d] : sA[d]) + rho[k] * g;
+                us[k][d] = u[d] + F * ir;  // Eq. 16: the shifted velocity
+            }
         }
     }
     // Eq. 5 factored per weight class c (0 rest, 1 axis, 2 diagonal) for the
@@ -999,9 +1049,15 @@ __device__ __forceinline__ void lean_site(const Lattice& L, const LeanShared<PRE
         C fp[2][2];
 #pragma unroll
         for (int k = 0; k < 2; k++) {
-            const C cu = along<C>(lo, us[k]), e = A[k][c] + (H[k][c] * cu) * cu;
-            fp[0][k] = e + B[k][c] * cu;
-            fp[1][k] = e - B[k][c] * cu;
+            const C cu = along<C>(lo, us[k]);
+            if constexpr (PREC == LB_FP64) {
+                const C e = A[k][c] + (H[k][c] * cu) * cu;
+                fp[0][k] = e + B[k][c] * cu;
+                fp[1][k] = e - B[k][c] * cu;
+            } else {
+                fp[0][k] = A[k][c] + cu * (B[k][c] + H[k][c] * cu);
+                fp[1][k] = A[k][c] - cu * (B[k][c] - H[k][c] * cu);
+            }
         }
 #pragma unroll
         for (int side = 0; side < 2; side++) {
