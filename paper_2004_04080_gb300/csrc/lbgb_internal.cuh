@@ -431,8 +431,8 @@ __device__ __forceinline__ void sc_force(const Lattice& L, const SiteNbr& n, con
             pb = pw[2 * (side * nxy + w) + 1];
         } else {
             long long m = nbr_index(L, n, i);
-            pa = __ldg(psi + 2 * m);
-            pb = __ldg(psi + 2 * m + 1);
+            pa = psi[2 * m];
+            pb = psi[2 * m + 1];
         }
         C w = wgt<C>(i);
         if (cx(i)) { sA[0] += C(cx(i)) * w * pa; sB[0] += C(cx(i)) * w * pb; }
@@ -493,16 +493,16 @@ __device__ __forceinline__ ParticleRef<C> particle_load(const Lattice& L, int p)
 #pragma unroll
     for (int d = 0; d < 3; d++) {
         if (sizeof(C) == 8) {
-            double q = __ldg(L.pos + 3 * p + d);
+            double q = L.pos[3 * p + d];
             r.ip[d] = (int)floor(q);
             r.fr[d] = C(q - (double)r.ip[d]);
-            r.v[d] = C(__ldg(L.vel + 3 * p + d));
-            r.w[d] = C(__ldg(L.omg + 3 * p + d));
+            r.v[d] = C(L.vel[3 * p + d]);
+            r.w[d] = C(L.omg[3 * p + d]);
         } else {
-            r.ip[d] = __ldg(L.ipos + 3 * p + d);
-            r.fr[d] = C(__ldg(L.fsnap + 9 * p + d));
-            r.v[d] = C(__ldg(L.fsnap + 9 * p + 3 + d));
-            r.w[d] = C(__ldg(L.fsnap + 9 * p + 6 + d));
+            r.ip[d] = L.ipos[3 * p + d];
+            r.fr[d] = C(L.fsnap[9 * p + d]);
+            r.v[d] = C(L.fsnap[9 * p + 3 + d]);
+            r.w[d] = C(L.fsnap[9 * p + 6 + d]);
         }
     }
     return r;
@@ -693,6 +693,10 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // every such kernel, lets the next one do the same and then waits until the
 // one before has ended and its writes are seen (each kernel of the chain waits
 // for its predecessor before it ends, so all earlier ones have ended too).
+// A kernel's lifetime then overlaps that of the kernel before it, so what that
+// one writes is not read-only for its lifetime: no kernel of a chain reads it
+// through the non-coherent path (ld.global.nc, which the compiler also takes for
+// pointers that are const and __restrict__, and which chain_begin does not order).
 // A call of one step at 32^3 FP32 83 -> 66 us, a step at 128^3 161 -> 149, at
 // 140x92x110 with unequal tau 255 -> 242, one adjoint gradient at 64^3 12.1 -> 10.8 ms.
 __device__ __forceinline__ void chain_begin() {

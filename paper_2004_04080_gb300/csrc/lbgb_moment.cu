@@ -718,7 +718,7 @@ __global__ void __launch_bounds__(128) k_bounce_links(const __grid_constant__ La
         float F[3] = {0, 0, 0}, T[3] = {0, 0, 0};
         if (k < n) {
             const unsigned* rec = seg + k;
-            auto get = [&]() { const unsigned v = __ldg(rec); rec += L.N; return v; };
+            auto get = [&]() { const unsigned v = *rec; rec += L.N; return v; };
             const unsigned s = get(), nbc = get(), bits = nbc & NB_LINKS;
             F2 h[3], r;
 #pragma unroll
