@@ -337,6 +337,8 @@ __device__ __forceinline__ void refill_node(const Lattice& L, long long s, int p
     for (int k = 0; k < 2; k++) rb[k] = den > C(0) ? num[k] / den : C(L.P.rho0[k]);
     if (MOM) {
         if (lane == 0) {
+            // (the density pass that would judge them is not run again)
+            if (!(rb[0] >= C(0) && rb[1] >= C(0) && rb[0] + rb[1] < C(1e30))) atomicOr(L.flags, FLAG_NONFINITE);
             for (int k = 0; k < 2; k++) ((C*)L.psi)[2 * s + k] = rb[k];
             for (int m = 0; m < 3; m++) ((C*)L.mom)[m * L.pstride + s] = (rb[0] + rb[1]) * uw[m];
         }

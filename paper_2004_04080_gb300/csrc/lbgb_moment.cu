@@ -107,6 +107,14 @@ __device__ __forceinline__ F2 rcp_newton(F2 x) {
     return fma2(fma2(f2(-1.f) * x, r, f2(1.f)), r, r);
 }
 
+// Densities of a step are judged where their sums are complete: by k_moments,
+// or, where links come back from particles or z faces, by the last of the
+// kernels that add these (k_bounce_links, k_moment_faces).
+template <int NK>
+__device__ __forceinline__ void check_density(const Lattice& L, float a, float b) {
+    if (NK == 2 ? !(a >= 0.f && b >= 0.f && a + b < 1e30f) : !(a > 0.f && a < 1e30f)) atomicOr(L.flags, FLAG_NONFINITE);
+}
+
 // ------------------------------------------------------------ the kernel
 // The two outer lanes on each side of a warp serve its neighbours only (the
 // sums S = sum_i w_i psi(x + c_i) c_i of a lane need the psi of the next one,
@@ -497,7 +505,9 @@ __global__ void __launch_bounds__(MNT, NK == 1 ? 4 : 3)
         copy.others(L, sh, z0, 0);
         cp_async_commit();
         Slots slot = {2, 0, 1};
-        unsigned solid = 0;  // particle nodes of the two sites: bits 0, 1 this plane, bits 2, 3 the one before
+        // of the two sites, bits 0, 1: without fluid, bits 2, 3: with links that
+        // come back from particles; the plane before it: bits 4 to 7
+        unsigned solid = 0;
         const long long seg = PART ? segment_of(L, x0, y0, H, z0, z1 - z0) : 0;
         const F2 zero = f2(0.f);
         MomentSum<NK> below, level;  // sums in progress of the plane before and of this one
@@ -516,7 +526,7 @@ __global__ void __launch_bounds__(MNT, NK == 1 ? 4 : 3)
                 F2 h[NK][3], r[NK], P[NK], r2[NK], r4[NK], P2[NK];
                 const unsigned off = me.collide(L, sh, slot.a, z, h, r, P);
                 if constexpr (PART) {
-                    solid = solid << 2 | off;
+                    solid = solid << 4 | off | (me.nbn[0] & NB_LINKS ? 4u : 0u) | (me.nbn[1] & NB_LINKS ? 8u : 0u);
                     if (z >= z0 && z < z1) {
                         const bool fr[2] = {own0 && !(off & 1u) && (me.nbn[0] & NB_LINKS),
                                             own1 && !(off & 2u) && (me.nbn[1] & NB_LINKS)};
@@ -665,19 +675,18 @@ __global__ void __launch_bounds__(MNT, NK == 1 ? 4 : 3)
             for (int d = 0; d < 3; d++) j[d] = fma2(j[d], f2(h36), j[d] * f2(l36));
             float* psi_z = psi_o + NK * nxy * (z - 1);
             float* mom_z = mom_o + nxy * (z - 1);
+            const bool face = !L.per[2] && (z == 1 || z == L.nz);  // plane z - 1 lies at a z face
 #pragma unroll
             for (int e = 0; e < 2; e++) {
                 if (!(e == 0 ? own0 : own1)) continue;
                 float ra = e == 0 ? lo(o[0]) : hi(o[0]), rb = e == 0 ? lo(o[NK - 1]) : hi(o[NK - 1]);
-                const bool off = PART && (solid & (e == 0 ? 4u : 8u));
+                const bool off = PART && (solid & (e == 0 ? 16u : 32u));
                 if (off) ra = rb = 0.f;
-                if (NK == 2) {
-                    if (!(ra >= 0.f && rb >= 0.f && ra + rb < 1e30f)) atomicOr(L.flags, FLAG_NONFINITE);
+                if (!face && !(PART && (solid & (e == 0 ? 64u : 128u)))) check_density<NK>(L, ra, rb);
+                if (NK == 2)
                     reinterpret_cast<float2*>(psi_z)[at[e]] = make_float2(ra, rb);
-                } else {
-                    if (!(ra > 0.f && ra < 1e30f)) atomicOr(L.flags, FLAG_NONFINITE);
+                else
                     psi_z[at[e]] = ra;
-                }
                 float* mz = mom_z;
 #pragma unroll
                 for (int d = 0; d < 3; d++) mz[at[e]] = off ? 0.f : (e == 0 ? lo(j[d]) : hi(j[d])), mz += ps;
@@ -838,7 +847,9 @@ __global__ void __launch_bounds__(128) k_bounce_links(const __grid_constant__ La
 #pragma unroll
             for (int d = 0; d < 3; d++) j[d] = fmaf((float)-nd[d], rr, j[d]);
             constexpr float h36 = 1.0f / 36.0f, l36 = (float)(1.0 / 36.0 - (double)h36);
-            *ps = fma2(back, f2(h36), fma2(back, f2(l36), sum));
+            const F2 full = fma2(back, f2(h36), fma2(back, f2(l36), sum));
+            *ps = full;
+            if (L.per[2] || (z > 0 && z < L.nz - 1)) check_density<2>(L, lo(full), hi(full));
 #pragma unroll
             for (int d = 0; d < 3; d++) *mo = fmaf(j[d], h36, fmaf(j[d], l36, js[d])), mo += L.pstride;
         }
@@ -914,13 +925,15 @@ __global__ void k_moment_faces(const __grid_constant__ Lattice L, float* __restr
     }
     // the reference fluid's links: weight 6 in all, along z only
     constexpr float h36 = 1.0f / 36.0f, l36 = (float)(1.0 / 36.0 - (double)h36);
-    float ref = 0;
+    float ref = 0, full[NK];
 #pragma unroll
     for (int k = 0; k < NK; k++) {
         add[k] += 6.f * L.rref[k];
         ref += 6.f * L.rref[k];
-        psi_o[NK * s + k] = fmaf(add[k], h36, fmaf(add[k], l36, psi_o[NK * s + k]));
+        full[k] = fmaf(add[k], h36, fmaf(add[k], l36, psi_o[NK * s + k]));
+        psi_o[NK * s + k] = full[k];
     }
+    check_density<NK>(L, full[0], full[NK - 1]);
     j[2] += face == 0 ? ref : -ref;
 #pragma unroll
     for (int d = 0; d < 3; d++) mom_o[d * L.pstride + s] = fmaf(j[d], h36, fmaf(j[d], l36, mom_o[d * L.pstride + s]));
