@@ -92,6 +92,7 @@ const int DOUBLES_PER_PARTICLE = 57;  // pos..Ttot, see carve()
 // sequence of rounding bits is fixed by it and the steps since lb_init_fields)
 const unsigned long long SR_DEFAULT_SEED = 0x2545F4914F6CDD1Dull;
 const int RED_BLOCKS = 1024;
+const size_t FLAG_BYTES = 64;  // the error flags and Lattice::spread
 const int PROF_MAX = 16384;
 
 struct Layout {
@@ -125,7 +126,7 @@ Layout layout(int nx, int ny, int nz, int prec, int maxc, int ncomp) {
     l.evt = off; off = align_up(off + (size_t)Np * 4);
     l.nb = off; off = align_up(off + (size_t)Np * 4);
     l.nb_chg = off; off = align_up(off + (size_t)(ncomp == 2 ? 8 + NB_CHG_CAP : 0) * 4);
-    l.flags = off; off = align_up(off + 64);
+    l.flags = off; off = align_up(off + FLAG_BYTES);
     int mc = maxc > 0 ? maxc : 1;
     l.col = off; off = align_up(off + (size_t)mc * DOUBLES_PER_PARTICLE * 8);
     l.prev = off; off = align_up(off + (size_t)mc * 4);
@@ -266,6 +267,8 @@ int lb_create(int nx, int ny, int nz, int prec, int max_colloids, void* d_worksp
     L.nb = (uint32_t*)(ctx->ws + l.nb);
     L.nb_chg = (int*)(ctx->ws + l.nb_chg);
     L.flags = (int*)(ctx->ws + l.flags);
+    L.spread = L.flags + 1;
+    L.turn = -1;
     int mc = max_colloids > 0 ? max_colloids : 1;
     double* c = (double*)(ctx->ws + l.col);
     double** slots3[] = {&L.pos, &L.vel, &L.omg};
@@ -303,7 +306,7 @@ int lb_create(int nx, int ny, int nz, int prec, int max_colloids, void* d_worksp
     cudaError_t e = cudaMemsetAsync(ctx->ws + l.mask, 0, Np, ctx->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(ctx->ws + l.owner, 0xff, Np * 4, ctx->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(ctx->ws + l.evt, 0, Np * 4, ctx->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(ctx->ws + l.flags, 0, 64, ctx->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(ctx->ws + l.flags, 0, FLAG_BYTES, ctx->stream);
     // psi: kernels read it on particle nodes that no virtual density has
     // reached yet (deep nodes), where any finite value serves
     if (e == cudaSuccess) e = cudaMemsetAsync(ctx->ws + l.psi, 0, 2 * Np * compute_bytes(prec), ctx->stream);
@@ -387,13 +390,14 @@ int lb_init_fields(lb_ctx* ctx, const double* rhoA, const double* rhoB, const do
     if (L.ncomp == 2) CK(cudaMemcpyAsync(st + L.N, rhoB, nb, cudaMemcpyHostToDevice, ctx->stream), "copy rhoB");
     if (u) CK(cudaMemcpyAsync(st + 2 * L.N, u, 3 * nb, cudaMemcpyHostToDevice, ctx->stream), "copy u");
     else CK(cudaMemsetAsync(st + 2 * L.N, 0, 3 * nb, ctx->stream), "zero u");
-    // any density near those of the fluid serves: the mean of some sites
+    // reference densities of the moment kernels: the mean of some sites
     const double* rho[2] = {rhoA, rhoB};
     for (int k = 0; k < L.ncomp; k++) {
         double sum = 0.0;
         const long long step = L.N / 1024 + 1, n = (L.N + step - 1) / step;
         for (long long s = 0; s < L.N; s += step) sum += rho[k][s];
-        L.rref[k] = isfinite((float)(sum / n)) ? (float)(sum / n) : 0.f;
+        L.rref[k] = isfinite((float)(sum / n)) ? fmaxf((float)(sum / n), 0.f) : 0.f;
+        L.rlow[k] = 0.5f * L.rref[k];
     }
     L.nc = 0;
     ctx->all_fixed = 1;
@@ -561,7 +565,7 @@ int lb_step(lb_ctx* ctx, int nsteps) {
     if (!ctx->have_fields) return set_err(ctx, LB_ERR_STATE, "lb_init_fields must come first");
     Lattice& L = ctx->L;
     cudaStream_t s = ctx->stream;
-    CK(cudaMemsetAsync(L.flags, 0, 4, s), "clear flags");
+    CK(cudaMemsetAsync(L.flags, 0, FLAG_BYTES, s), "clear flags");
     MomentRun run = moment_run(ctx, nsteps);
     Lattice V = L;  // the view the kernels get: psi and mom of the present time
     for (int t = 0; L.ncomp == 1 && t < nsteps; t++) {
@@ -575,6 +579,7 @@ int lb_step(lb_ctx* ctx, int nsteps) {
         if (run.on) {
             V.psi = run.psi[0];
             V.mom = run.mom[0];
+            V.turn = t % 3;
             if (t == 0) {
                 if (int rc = prof_mark(ctx, LB_KERNEL_DENSITY, 0, s)) return rc;
                 n += launch_single_moments(V, ctx->prec, s);
@@ -635,6 +640,7 @@ int lb_step(lb_ctx* ctx, int nsteps) {
         if (run.on) {
             V.psi = run.psi[0];
             V.mom = run.mom[0];
+            V.turn = t % 3;
         }
         n += launch_remap(V, ctx->prec, kept, t == 0, s);  // destroy / create (Eqs. 24, 25)
         if (L.nc > 0) {

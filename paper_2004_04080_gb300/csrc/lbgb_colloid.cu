@@ -163,12 +163,13 @@ __device__ __forceinline__ typename Prec<PREC>::C node_rho(const Lattice& L, lon
     return site_rho<PREC>(L, s, k);
 }
 
-// a node a particle covers holds no fluid (MOM: the density pass is not run again)
+// a node a particle covers holds no fluid (MOM: the density pass is not run
+// again), but a density of use to k_moments
 template <int PREC, bool MOM>
 __device__ __forceinline__ void clear_moments(const Lattice& L, long long s) {
     typedef typename Prec<PREC>::C C;
     if (MOM) {
-        for (int k = 0; k < 2; k++) ((C*)L.psi)[2 * s + k] = C(0);
+        for (int k = 0; k < 2; k++) ((C*)L.psi)[2 * s + k] = C(L.rref[k]);
         for (int d = 0; d < 3; d++) ((C*)L.mom)[d * L.pstride + s] = C(0);
     }
 }
@@ -337,8 +338,7 @@ __device__ __forceinline__ void refill_node(const Lattice& L, long long s, int p
     for (int k = 0; k < 2; k++) rb[k] = den > C(0) ? num[k] / den : C(L.P.rho0[k]);
     if (MOM) {
         if (lane == 0) {
-            // (the density pass that would judge them is not run again)
-            if (!(rb[0] >= C(0) && rb[1] >= C(0) && rb[0] + rb[1] < C(1e30))) atomicOr(L.flags, FLAG_NONFINITE);
+            if (rb[0] < C(L.rlow[0]) || rb[1] < C(L.rlow[1])) note_spread(L, L.turn);
             for (int k = 0; k < 2; k++) ((C*)L.psi)[2 * s + k] = rb[k];
             for (int m = 0; m < 3; m++) ((C*)L.mom)[m * L.pstride + s] = (rb[0] + rb[1]) * uw[m];
         }

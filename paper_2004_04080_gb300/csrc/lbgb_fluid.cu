@@ -38,8 +38,9 @@ __global__ void k_init(Lattice L, const double* __restrict__ stage) {
 // rho^k on fluid nodes (0 on particle nodes) into psi; flags non-finite or
 // negative densities.  MOM: also the total momentum j^A + j^B (Eq. 7) into
 // the rows mom[d][s] (0 on particle nodes), for the omega = 1 collision: with
-// tau_A = tau_B the mixture velocity (Eq. 14) needs only the sum.
-template <int PREC, bool MOM>
+// tau_A = tau_B the mixture velocity (Eq. 14) needs only the sum.  KEEP: the
+// first step of a call that keeps moments.
+template <int PREC, bool MOM, bool KEEP>
 __global__ void k_density(Lattice L) {
     chain_begin();
     typedef typename Prec<PREC>::S S;
@@ -49,8 +50,8 @@ __global__ void k_density(Lattice L) {
     C* psi = (C*)L.psi;
     C* mom = (C*)L.mom;
     if (L.mask[s]) {
-        psi[2 * s] = 0;
-        psi[2 * s + 1] = 0;
+        psi[2 * s] = KEEP ? C(L.rref[0]) : C(0);  // (any density, of use to k_moments)
+        psi[2 * s + 1] = KEEP ? C(L.rref[1]) : C(0);
         if (MOM)
 #pragma unroll
             for (int a = 0; a < 3; a++) mom[a * L.pstride + s] = 0;
@@ -96,6 +97,7 @@ __global__ void k_density(Lattice L) {
         for (int d = 0; d < 3; d++) mom[d * L.pstride + s] = jt[d];
     if (!(rho[0] >= C(0) && rho[1] >= C(0) && rho[0] < C(1e30) && rho[1] < C(1e30)))
         atomicOr(L.flags, FLAG_NONFINITE);
+    if (KEEP && (rho[0] < C(L.rlow[0]) || rho[1] < C(L.rlow[1]))) note_spread(L, L.turn);
 }
 
 // wall density ("wetting mode 0"): w_i-weighted mean density of the fluid
@@ -917,6 +919,10 @@ __device__ __forceinline__ void lean_site(const Lattice& L, const LeanShared<PRE
     C rho[2];
 #pragma unroll
     for (int k = 0; k < 2; k++) rho[k] = solid ? prm<C>(L.P.rho0[k], L.PF.rho0[k]) : sh.psi[sl[1]][1][tx + 1][k];
+    // (densities of the last step of a call that kept moments are judged here;
+    // FP64 densities come from the density pass, which has judged them)
+    if (PREC != LB_FP64 && !solid && !(rho[0] >= C(0) && rho[1] >= C(0) && rho[0] < C(1e30) && rho[1] < C(1e30)))
+        atomicOr(L.flags, FLAG_NONFINITE);
     C us[2][3];
     // FP64, which the operations bound: by opposite pairs and without divisions.
     // FP32 and FP16 sum link by link (see k_density: the same last bits)
@@ -1499,10 +1505,13 @@ int launch_init_fields(const Lattice& L, int prec, const double* stage, cudaStre
 }
 
 int launch_density(const Lattice& L, int prec, cudaStream_t st) {
-    if (L.dense_mom) {
-        DISPATCH(prec, (launch_after(k_density<P, true>, nblk(L.N, 256), 256, 0, st, L)));
+    if (L.turn >= 0) {  // (FP32 arithmetic)
+        if (prec == LB_FP16) launch_after(k_density<LB_FP16, true, true>, nblk(L.N, 256), 256, 0, st, L);
+        else launch_after(k_density<LB_FP32, true, true>, nblk(L.N, 256), 256, 0, st, L);
+    } else if (L.dense_mom) {
+        DISPATCH(prec, (launch_after(k_density<P, true, false>, nblk(L.N, 256), 256, 0, st, L)));
     } else {
-        DISPATCH(prec, (launch_after(k_density<P, false>, nblk(L.N, 256), 256, 0, st, L)));
+        DISPATCH(prec, (launch_after(k_density<P, false, false>, nblk(L.N, 256), 256, 0, st, L)));
     }
     return 1;
 }

@@ -260,6 +260,10 @@ struct Lattice {
     int tau_equal;     // tau_A == tau_B
     ParamsF PF;        // FP32 copies (see ParamsF)
     float rref[2];     // about the mean initial density: the moment kernel sums deviations from it
+    float rlow[2];     // half of it
+    int* spread;       // [3], in the steps of a call that go from moments to moments, cleared at its start:
+    int turn;          // entry turn = t mod 3 (-1 in other calls) says whether the density pass or the step
+                       // before has met a density below rlow; the step then sums without a reference
     int* ipos;         // [n][3] floor of the position (FP32 geometry origin)
     float* fsnap;      // [n][9] position - ipos, v(t-1/2), omega(t-1/2) in FP32
     double* red;       // reduction partials
@@ -670,6 +674,11 @@ __device__ __forceinline__ void add_runs(const Lattice& L, int term, int p, cons
 __device__ __forceinline__ double acc_value(const Lattice& L, const unsigned long long* a) {
     if (!L.acc_wide) return (double)(long long)a[0] * 9.094947017729282e-13;  // 2^-40
     return (double)(long long)a[0] * 5.9604644775390625e-08 + (double)a[1] * 5.421010862427522e-20;
+}
+
+// a density below L.rlow was met
+__device__ __forceinline__ void note_spread(const Lattice& L, int turn) {
+    if (L.spread[turn] == 0) L.spread[turn] = 1;
 }
 
 // asynchronous global -> shared copies (cp.async) and their completion

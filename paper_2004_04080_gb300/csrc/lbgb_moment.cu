@@ -40,12 +40,22 @@
 // particles 512 x 512 x 256 at a volume fraction of 0.15 (k_moments and
 // k_bounce_links) 4.12 -> 1.77 ms.
 //
-// The
-// links are summed as deviations from those of a fluid of a reference density
-// at rest (P less that density, L.rref): the sums of rho and j then stay small
-// and keep the precision that sums of the links themselves lose (a
-// run of 100 steps: a third of the rounding error of j of the populations'
-// sums, and no drift of the mass).
+// The links are summed as deviations from those of a fluid of a reference
+// density at rest (P less that density).  Where the densities are nearly uniform
+// the reference is their mean initial value: the sums of rho and j then stay
+// small and keep the precision that sums of the links themselves lose (48 x 40 x
+// 36, deviations of 1 %, 100 steps: the rms error of rho 1.0e-7 against 1.3e-7
+// by sums of the links and 1.6e-6 by sums of populations, of u 5e-9, 8e-9, 1.3e-8).
+// A density far below the reference would be left with the rounding of the
+// reference (0: with a residue of either sign).  So the references of a step are
+// 0 once the step before, or the density pass, has met a density below half of
+// them (L.spread; a site keeps its rest population, so that a density falls by
+// a factor of about 3 at most meanwhile): the sums of the links are each rounded
+// by their own size, and a component that is absent adds up to 0.  In slabs and
+// droplets of 0, 1e-4, 1e-2 and 0.05 against 0.7 to 1.3 the rms errors are then
+// those of sums of populations divided by 1.25 after 2 steps, 2.5 after 20, 7 after
+// 100, 30 after 1000 (rho, each relative to itself) and 1.25, 2.2, 2.0, 1.4 (u;
+// geometric means over 9 such states).
 #include "lbgb_internal.cuh"
 
 namespace lbgb {
@@ -107,14 +117,6 @@ __device__ __forceinline__ F2 rcp_newton(F2 x) {
     return fma2(fma2(f2(-1.f) * x, r, f2(1.f)), r, r);
 }
 
-// Densities of a step are judged where their sums are complete: by k_moments,
-// or, where links come back from particles or z faces, by the last of the
-// kernels that add these (k_bounce_links, k_moment_faces).
-template <int NK>
-__device__ __forceinline__ void check_density(const Lattice& L, float a, float b) {
-    if (NK == 2 ? !(a >= 0.f && b >= 0.f && a + b < 1e30f) : !(a > 0.f && a < 1e30f)) atomicOr(L.flags, FLAG_NONFINITE);
-}
-
 // ------------------------------------------------------------ the kernel
 // The two outer lanes on each side of a warp serve its neighbours only (the
 // sums S = sum_i w_i psi(x + c_i) c_i of a lane need the psi of the next one,
@@ -129,8 +131,9 @@ constexpr int MNT = 32 * (MW + 1);  // the warps of the rows and one for the row
 constexpr int MREC = 10;
 struct LinkList {
     unsigned* rec;  // [MREC][N]
-    int* count;     // per block
+    int* count;     // per block; with LIST_PLAIN if the step sums without a reference
 };
+constexpr int LIST_PLAIN = 1 << 30;
 // first entry of the segment of the block at (x0, y0, z0) with H rows and nz planes
 __device__ __forceinline__ long long segment_of(const Lattice& L, int x0, int y0, int H, int z0, int nz) {
     return (long long)L.nx * L.ny * z0 + (long long)nz * ((long long)y0 * L.nx + (long long)H * x0);
@@ -150,7 +153,8 @@ struct alignas(16) MomentShared {
     // each side, of the plane in use and the next two, and the link classes
     float own[3][NK == 2 ? 3 : 4][MROWS + 2][32];
     uint32_t nb[PART ? 3 : 1][PART ? MROWS + 2 : 1][PART ? 32 : 1];
-    int count;  // boundary sites listed so far
+    float ref[NK];  // reference densities of the step
+    int count;      // boundary sites listed so far
 };
 
 // the links along +c and -c of weight 1/36 (r2 = 2 rho) or 1/18 (r2 = 4 rho,
@@ -277,6 +281,9 @@ template <int NK, bool PART>
 struct MomentLane {
     int lane, row[2];  // rows of the block (1: the first)
     uint32_t nbn[2];   // link classes of the plane
+    // of the densities met: the signs of their distances above L.rlow (any site),
+    // and the largest as bits, which a negative one or no number exceeds (fluid)
+    unsigned below, top;
     PsiMarch march[2];
 
     __device__ __forceinline__ void place(int l, int ra, int rb) {
@@ -287,6 +294,7 @@ struct MomentLane {
 #pragma unroll
         for (int r = 0; r < 2; r++) march[r] = {zero, zero, zero, zero, zero, zero, zero};
         nbn[0] = nbn[1] = 0;
+        below = top = 0;
     }
     // with the psi plane of a slot: S of the plane before it, by row and component
     __device__ __forceinline__ void advance(const MomentShared<NK, PART>& sh, int slot, float (&S)[2][2][3]) {
@@ -302,6 +310,30 @@ struct MomentLane {
             }
             psi_march(march[r], p, S[r][0], S[r][1]);
         }
+    }
+    // The densities of a step are judged here, where k_moments reads them (those
+    // of the last step of a call by the kernel that pushes the populations): all
+    // links that came back from particles and faces are in them by now.
+    // What is below L.rlow is looked for by each warp among its sites, or, with
+    // particles, by the ring warp in the staged psi of plane z + 1, where the march
+    // of the others has no register to spare.  (256^3 without and with 2407
+    // particles: k_moments 327 -> 326 and 372 -> 377 us a step; with a branch
+    // for the unusual densities, or their smallest ones kept, 331 to 345 and 392 to 402.)
+    __device__ __forceinline__ void meet(F2 d) { below |= __float_as_uint(lo(d)) | __float_as_uint(hi(d)); }
+    __device__ __forceinline__ void meet_rows(const Lattice& L, const MomentShared<NK, PART>& sh, int slot, int H) {
+        if constexpr (NK == 2)
+            for (int y = 0; y < H; y++) meet(sh.psi[slot][y + 2][lane] - f2(L.rlow[0], L.rlow[1]));
+    }
+    __device__ __forceinline__ void judge(const F2 (&r)[NK]) {
+        const unsigned none = NK == 1 ? 1u : 0u;  // one component: 0 is no density
+#pragma unroll
+        for (int k = 0; k < NK; k++)
+            top = max(top, max(__float_as_uint(lo(r[k])) - none, __float_as_uint(hi(r[k])) - none));
+    }
+    // what the lanes `own` have met
+    __device__ __forceinline__ void report(const Lattice& L, bool own) const {
+        if (__any_sync(0xffffffffu, own && (below >> 31)) && lane == 0) note_spread(L, L.turn == 2 ? 0 : L.turn + 1);
+        if (__any_sync(0xffffffffu, own && top >= __float_as_uint(1e30f)) && lane == 0) atomicOr(L.flags, FLAG_NONFINITE);
     }
     // h, rho and P of the sites of plane z, from the psi of plane z + 1 and the
     // other arrays of plane z in a slot; off: bits of the sites without fluid
@@ -319,6 +351,7 @@ struct MomentLane {
         if constexpr (NK == 2) {
             r[0] = f2(lo(march[0].p), lo(march[1].p));
             r[1] = f2(hi(march[0].p), hi(march[1].p));
+            if (!PART) meet(r[0] - f2(L.rlow[0])), meet(r[1] - f2(L.rlow[1]));
             if (PART) {
                 r[0] = f2(off & 1u ? 0.f : lo(r[0]), off & 2u ? 0.f : hi(r[0]));
                 r[1] = f2(off & 1u ? 0.f : lo(r[1]), off & 2u ? 0.f : hi(r[1]));
@@ -326,7 +359,9 @@ struct MomentLane {
             rt = r[0] + r[1];
         } else {
             r[0] = rt = both(NK == 1 ? 3 : 0);
+            meet(r[0] - f2(L.rlow[0]));
         }
+        if (!out) judge(r);
         if (PART) rt = f2(off & 1u ? 1.f : lo(rt), off & 2u ? 1.f : hi(rt));
         if (out) {
 #pragma unroll
@@ -353,7 +388,7 @@ struct MomentLane {
 #pragma unroll
         for (int k = 0; k < NK; k++) {
             const F2 hh = fma2(h[k][2], h[k][2], fma2(h[k][1], h[k][1], h[k][0] * h[k][0]));
-            P[k] = fma2(r[k] * hh, f2(-2.f / 3.f), r[k] - f2(L.rref[k]));
+            P[k] = fma2(r[k] * hh, f2(-2.f / 3.f), r[k] - f2(sh.ref[k]));
         }
         return off;
     }
@@ -415,6 +450,9 @@ __global__ void __launch_bounds__(MNT, NK == 1 ? 4 : 3)
     // and -1
     const int nw = (H + 1) / 2;
     if (PART && threadIdx.x == 0) sh.count = 0;
+    const bool plain = L.spread[L.turn];
+    if (threadIdx.x < NK) sh.ref[threadIdx.x] = plain ? 0.f : L.rref[threadIdx.x];
+    if (threadIdx.x == 0 && (blockIdx.x | blockIdx.y | blockIdx.z) == 0) L.spread[L.turn == 0 ? 2 : L.turn - 1] = 0;
     // psi of the planes z0 - 2 .. z0 and the other arrays of plane z0 - 1; the
     // slots go round with the planes
     PlaneCopy<NK, PART> copy;
@@ -442,6 +480,7 @@ __global__ void __launch_bounds__(MNT, NK == 1 ? 4 : 3)
             copy.psi(L, sh, min(z + 3, z1 + 1), slot.c);
             copy.others(L, sh, min(z + 2, z1), slot.c);
             cp_async_commit();
+            if (PART && !beyond(L, z + 1)) me.meet_rows(L, sh, slot.a, H);
             me.collide(L, sh, slot.a, z, h, r, P);
 #pragma unroll
             for (int k = 0; k < NK; k++) {
@@ -473,6 +512,7 @@ __global__ void __launch_bounds__(MNT, NK == 1 ? 4 : 3)
             block_barrier();
         }
         cp_async_wait_all();
+        if (PART) me.report(L, true);
     } else if (warp >= nw) {
         block_barrier();
         copy.psi(L, sh, z0 + 1, 0);
@@ -505,9 +545,7 @@ __global__ void __launch_bounds__(MNT, NK == 1 ? 4 : 3)
         copy.others(L, sh, z0, 0);
         cp_async_commit();
         Slots slot = {2, 0, 1};
-        // of the two sites, bits 0, 1: without fluid, bits 2, 3: with links that
-        // come back from particles; the plane before it: bits 4 to 7
-        unsigned solid = 0;
+        unsigned solid = 0;  // particle nodes of the two sites: bits 0, 1 this plane, bits 2, 3 the one before
         const long long seg = PART ? segment_of(L, x0, y0, H, z0, z1 - z0) : 0;
         const F2 zero = f2(0.f);
         MomentSum<NK> below, level;  // sums in progress of the plane before and of this one
@@ -526,7 +564,7 @@ __global__ void __launch_bounds__(MNT, NK == 1 ? 4 : 3)
                 F2 h[NK][3], r[NK], P[NK], r2[NK], r4[NK], P2[NK];
                 const unsigned off = me.collide(L, sh, slot.a, z, h, r, P);
                 if constexpr (PART) {
-                    solid = solid << 4 | off | (me.nbn[0] & NB_LINKS ? 4u : 0u) | (me.nbn[1] & NB_LINKS ? 8u : 0u);
+                    solid = solid << 2 | off;
                     if (z >= z0 && z < z1) {
                         const bool fr[2] = {own0 && !(off & 1u) && (me.nbn[0] & NB_LINKS),
                                             own1 && !(off & 2u) && (me.nbn[1] & NB_LINKS)};
@@ -670,19 +708,17 @@ __global__ void __launch_bounds__(MNT, NK == 1 ? 4 : 3)
             // alone would let the sums grow by 2e-8 a step
             constexpr float h36 = 1.0f / 36.0f, l36 = (float)(1.0 / 36.0 - (double)h36);
 #pragma unroll
-            for (int k = 0; k < NK; k++) o[k] = fma2(o[k], f2(h36), o[k] * f2(l36)) + f2(L.rref[k]);
+            for (int k = 0; k < NK; k++) o[k] = fma2(o[k], f2(h36), o[k] * f2(l36)) + f2(sh.ref[k]);
 #pragma unroll
             for (int d = 0; d < 3; d++) j[d] = fma2(j[d], f2(h36), j[d] * f2(l36));
             float* psi_z = psi_o + NK * nxy * (z - 1);
             float* mom_z = mom_o + nxy * (z - 1);
-            const bool face = !L.per[2] && (z == 1 || z == L.nz);  // plane z - 1 lies at a z face
 #pragma unroll
             for (int e = 0; e < 2; e++) {
                 if (!(e == 0 ? own0 : own1)) continue;
                 float ra = e == 0 ? lo(o[0]) : hi(o[0]), rb = e == 0 ? lo(o[NK - 1]) : hi(o[NK - 1]);
-                const bool off = PART && (solid & (e == 0 ? 16u : 32u));
-                if (off) ra = rb = 0.f;
-                if (!face && !(PART && (solid & (e == 0 ? 64u : 128u)))) check_density<NK>(L, ra, rb);
+                const bool off = PART && (solid & (e == 0 ? 4u : 8u));
+                if (off) ra = L.rref[0], rb = L.rref[NK - 1];  // (any density that is not below L.rlow)
                 if (NK == 2)
                     reinterpret_cast<float2*>(psi_z)[at[e]] = make_float2(ra, rb);
                 else
@@ -693,10 +729,11 @@ __global__ void __launch_bounds__(MNT, NK == 1 ? 4 : 3)
             }
         }
         cp_async_wait_all();
+        me.report(L, cols);
     }
     if constexpr (PART) {
         block_barrier();
-        if (threadIdx.x == 0) list.count[blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z)] = sh.count;
+        if (threadIdx.x == 0) list.count[blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z)] = sh.count | (plain ? LIST_PLAIN : 0);
     }
 }
 
@@ -718,7 +755,11 @@ __global__ void __launch_bounds__(128) k_bounce_links(const __grid_constant__ La
                                                        int parts, long long unit) {
     chain_begin();
     const int bx = blockIdx.x / parts, z0 = blockIdx.z * zc, x0 = bx * TW, y0 = blockIdx.y * MROWS;
-    const int n = list.count[bx + gridDim.x / parts * (blockIdx.y + gridDim.y * blockIdx.z)];
+    const int count = list.count[bx + gridDim.x / parts * (blockIdx.y + gridDim.y * blockIdx.z)];
+    const int n = count & ~LIST_PLAIN;
+    const bool plain = count & LIST_PLAIN;
+    const F2 ref = plain ? f2(0.f) : f2(L.rref[0], L.rref[1]);
+    if (plain) unit = 0;
     const unsigned* seg = list.rec + segment_of(L, x0, y0, min(MROWS, L.ny - y0), z0, min(zc, L.nz - z0));
     const int lane = threadIdx.x & 31, nx = L.nx, nxy = L.nx * L.ny;
     for (int k0 = (int)(blockIdx.x % parts * 128 + threadIdx.x) - lane; k0 < n; k0 += 128 * parts) {
@@ -753,7 +794,7 @@ __global__ void __launch_bounds__(128) k_bounce_links(const __grid_constant__ La
                                               (az > 0 ? dzp : (az < 0 ? dzm : 0)))];
             };
             // (as in k_moments, deviations from a fluid of the reference density at rest)
-            const F2 hh = fma2(h[2], h[2], fma2(h[1], h[1], h[0] * h[0])), ref = f2(L.rref[0], L.rref[1]);
+            const F2 hh = fma2(h[2], h[2], fma2(h[1], h[1], h[0] * h[0]));
             const F2 P = fma2(r * hh, f2(-2.f / 3.f), r - ref), P2 = P + P, r2 = r + r, r4 = r2 + r2;
             F2 back = f2(0.f);
             float j[3] = {0, 0, 0};
@@ -785,7 +826,7 @@ __global__ void __launch_bounds__(128) k_bounce_links(const __grid_constant__ La
                 nd[d] = __popc(bits & up) - __popc(bits & dn) + 2 * (int)((bits >> (2 * d + 1)) & 1u) -
                         2 * (int)((bits >> (2 * d + 2)) & 1u);
             }
-            const float rr = L.rref[0] + L.rref[1];
+            const float rr = lo(ref) + hi(ref);
             float U[3], rel[3];
             if (nbc & NB_MULTI) {
                 // next to two particles: each link with its own, forces added directly
@@ -847,9 +888,7 @@ __global__ void __launch_bounds__(128) k_bounce_links(const __grid_constant__ La
 #pragma unroll
             for (int d = 0; d < 3; d++) j[d] = fmaf((float)-nd[d], rr, j[d]);
             constexpr float h36 = 1.0f / 36.0f, l36 = (float)(1.0 / 36.0 - (double)h36);
-            const F2 full = fma2(back, f2(h36), fma2(back, f2(l36), sum));
-            *ps = full;
-            if (L.per[2] || (z > 0 && z < L.nz - 1)) check_density<2>(L, lo(full), hi(full));
+            *ps = fma2(back, f2(h36), fma2(back, f2(l36), sum));
 #pragma unroll
             for (int d = 0; d < 3; d++) *mo = fmaf(j[d], h36, fmaf(j[d], l36, js[d])), mo += L.pstride;
         }
@@ -891,6 +930,7 @@ __global__ void k_moment_faces(const __grid_constant__ Lattice L, float* __restr
     }
     const float* uw = face == 0 ? L.PF.wall_u_lo : L.PF.wall_u_hi;
     const int type = L.P.open[face];
+    const bool plain = L.spread[L.turn];
     const bool ext = L.P.open_extrap && (type == 1 || type == 2);
     // the face values of the column (k_face_values): rho_w^k, u_w
     const float* fv = (const float*)L.face + 5 * ((long long)face * L.nx * L.ny + xy);
@@ -910,7 +950,7 @@ __global__ void k_moment_faces(const __grid_constant__ Lattice L, float* __restr
             const float cs = cx(i) * us[k][0] + cy(i) * us[k][1] + az * us[k][2];
             const float ss = us[k][0] * us[k][0] + us[k][1] * us[k][1] + us[k][2] * us[k][2];
             // less the link of the reference fluid (see k_moments), in units of 1/36
-            const float W = i <= 6 ? 2.f : 1.f, ref = L.rref[k], ro = (float)L.P.open_rho[face][k];
+            const float W = i <= 6 ? 2.f : 1.f, ref = plain ? 0.f : L.rref[k], ro = (float)L.P.open_rho[face][k];
             const float fs = W * ((rho[k] - ref) + rho[k] * (3.f * cs + 4.5f * cs * cs - 1.5f * ss));
             float fb;
             if (type == 1) fb = W * (2.f * (ro - ref) + ro * (9.f * cu * cu - 3.f * uu)) - fs;
@@ -925,15 +965,13 @@ __global__ void k_moment_faces(const __grid_constant__ Lattice L, float* __restr
     }
     // the reference fluid's links: weight 6 in all, along z only
     constexpr float h36 = 1.0f / 36.0f, l36 = (float)(1.0 / 36.0 - (double)h36);
-    float ref = 0, full[NK];
+    float ref = 0;
 #pragma unroll
     for (int k = 0; k < NK; k++) {
-        add[k] += 6.f * L.rref[k];
-        ref += 6.f * L.rref[k];
-        full[k] = fmaf(add[k], h36, fmaf(add[k], l36, psi_o[NK * s + k]));
-        psi_o[NK * s + k] = full[k];
+        add[k] += plain ? 0.f : 6.f * L.rref[k];
+        ref += plain ? 0.f : 6.f * L.rref[k];
+        psi_o[NK * s + k] = fmaf(add[k], h36, fmaf(add[k], l36, psi_o[NK * s + k]));
     }
-    check_density<NK>(L, full[0], full[NK - 1]);
     j[2] += face == 0 ? ref : -ref;
 #pragma unroll
     for (int d = 0; d < 3; d++) mom_o[d * L.pstride + s] = fmaf(j[d], h36, fmaf(j[d], l36, mom_o[d * L.pstride + s]));

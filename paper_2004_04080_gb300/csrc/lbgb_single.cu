@@ -81,6 +81,7 @@ __global__ void k1_density(Lattice L) {
         if (cz(i)) j[2] += C(cz(i)) * v;
     }
     if (!(rho > C(0) && rho < C(1e30))) atomicOr(L.flags, FLAG_NONFINITE);
+    if (rho < C(L.rlow[0])) note_spread(L, L.turn);
     ((C*)L.psi)[s] = rho;
 #pragma unroll
     for (int d = 0; d < 3; d++) ((C*)L.mom)[d * L.pstride + s] = j[d];
