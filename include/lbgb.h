@@ -286,7 +286,9 @@ int lb_drag_gradient(lb_ctx *ctx, const double *d_F, double weight, double eps, 
 /* Record during the next nsteps time steps of lb_step: the populations f(t)
  * at the start of each step into d_states (consecutive blocks of
  * lb_state_bytes) and the link forces F_liq (Eq. 22) after each step into
- * d_forces ([nsteps][n][3] doubles); either may be NULL.  Device-to-device
+ * d_forces ([nsteps][n][3] doubles); either may be NULL.  The recorded steps
+ * store the populations of every step (see lb_step), with both pointers NULL
+ * too, so that a run recorded in part is repeated bit for bit.  Device-to-device
  * copies on the context stream, so a checkpointed reverse sweep needs no host
  * round trip per step.  nsteps <= 0 stops a recording. */
 int lb_record(lb_ctx *ctx, void *d_states, double *d_forces, int nsteps);

@@ -71,8 +71,10 @@ class AdjointRunner:
         for start in range(0, self.steps, self.K):
             self.checkpoints[start] = self._state()
             m = min(self.K, self.steps - start)
-            if self.n:
-                lbgb.lb_record(lat.h, None, forces[start].data_ptr(), m)
+            # recorded steps go from populations to populations, as those that the
+            # reverse sweep recomputes (a call that does not record may keep
+            # moments between its steps, which rounds differently)
+            lbgb.lb_record(lat.h, None, forces[start].data_ptr() if self.n else None, m)
             lat.step(m)
         self.checkpoints[self.steps] = self._state()
         J = 0.0
