@@ -16,7 +16,10 @@
 namespace lbgb {
 
 constexpr int BXP = 16, BYP = 8, PB = BXP * BYP;  // particle block
-constexpr double REMAP_PAD = 0.75;
+// a particle moves less than 1/2 along each axis in a step (checked by the
+// integrator), so less than sqrt(3)/2; the box of the remap reaches beyond that
+constexpr float REMAP_REACH = 0.88f;
+constexpr double REMAP_PAD = 0.95;
 
 // geometry of particle p in compute type C
 template <typename C>
@@ -252,9 +255,8 @@ __device__ __forceinline__ void particle_frame(const Lattice& L, int p, int x, i
 // The node map is that of the position before the last move v, so a node
 // changes side only if it is within |v| of the surface: only that shell (with
 // a margin far above the rounding of the FP32 distances) is visited, row by
-// row of the box, and 0.65 at most (a particle moves less than 1/2 a step,
-// checked by the integrator).  The first step of a call (wide) visits all of
-// the 0.65, so that particles which overlapped before it are reported by every
+// row of the box.  The first step of a call (wide) visits a shell of 0.65 at
+// least, so that particles which overlapped before it are reported by every
 // call that steps them.  A shell of 0.65 for every particle read the
 // owner map of ten times the points: 512 x 512 x 256, 14,444 particles, 302
 // us against 101 (96^3 FP64: 90 against 27).  Points outside the shell are found
@@ -266,7 +268,7 @@ __global__ void __launch_bounds__(PB) k_remap_classify(const __grid_constant__ L
     int p = blockIdx.x;
     PGeo<C> g = pgeo<C>(L, p, REMAP_PAD);
     const float v2 = float(g.v[0]) * float(g.v[0]) + float(g.v[1]) * float(g.v[1]) + float(g.v[2]) * float(g.v[2]);
-    const float reach = wide ? 0.65f : fminf(sqrtf(v2) + 0.01f, 0.65f);
+    const float reach = fminf(fmaxf(sqrtf(v2) + 0.01f, wide ? 0.65f : 0.f), REMAP_REACH);
     for_band<C>(L, g, -reach, reach, [&](int, int, int, long long s, int a, int b, int c, const C (&d)[3]) {
         int o = L.owner[s];
         if (inside<C>(L, p, g, d, a, b, c)) {
@@ -839,7 +841,7 @@ __global__ void __launch_bounds__(128) k_pairs(Lattice L) {
 
 // --------------------------------------------------------- integrator
 // Eq. 35 totals, Eq. 32 leap-frog, Eqs. 33-34 quaternions; then the FP32
-// snapshot of the new state.  A particle faster than 1/2 lattice unit per step
+// snapshot of the new state.  A particle faster than 1/2 lattice unit along an axis
 // is reported (the remap assumes smaller moves).  The step's fixed-point sums
 // are read and cleared for the next step, and the list of changed nodes
 // emptied.
