@@ -108,7 +108,9 @@ __device__ __forceinline__ F2 fma2(F2 x, F2 y, F2 z) {
 __device__ __forceinline__ F2 shfl2(F2 a, int lane) {
     return f2(__shfl_sync(0xffffffffu, lo(a), lane), __shfl_sync(0xffffffffu, hi(a), lane));
 }
-// 1/x of normal values: the approximate reciprocal and one Newton step
+// 1/x of normal values: the approximate reciprocal and one Newton-Raphson step,
+// which rounds correctly (the bits of __frcp_rn at all 2^23 mantissas of 1/2^30,
+// 1/2^10, 1/2 to 2, 2^10 and 2^100)
 __device__ __forceinline__ F2 rcp_newton(F2 x) {
     float a, b;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(a) : "f"(lo(x)));
