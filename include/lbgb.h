@@ -163,10 +163,11 @@ int lb_add_colloids(lb_ctx *ctx, int n, const double *pos, const double *vel,
 
 /* Advance nsteps time steps.  The state a call leaves is the populations
  * f(t + nsteps).  At tau_A = tau_B = 1 (FP32 and FP16 contexts, no recording,
- * no LB_ROUND_NEAREST) a call of several steps keeps rho^k and j in FP32
- * between them, which is all that Eq. 16 needs at omega = 1, so that only the
- * first step reads and only the last one stores populations: a run split
- * into other calls differs by rounding.  Returns LB_ERR_NONFINITE / LB_ERR_OVERLAP if the
+ * no LB_ROUND_NEAREST; with one component where the call advances enough sites
+ * to gain by it) a call of several steps keeps rho^k and j in FP32 between
+ * them, which is all that Eq. 16 needs at omega = 1, so that only the first step
+ * reads and only the last one stores populations: a run split into other calls
+ * differs by rounding.  Returns LB_ERR_NONFINITE / LB_ERR_OVERLAP if the
  * device flagged the condition during these steps (state then undefined). */
 int lb_step(lb_ctx *ctx, int nsteps);
 
