@@ -542,13 +542,8 @@ static MomentRun moment_run(const lb_ctx* ctx, int nsteps) {
     // that a run of moments starts with a kernel more (4 us) and moves a fifth of
     // the bytes afterwards, which small lattices do not wait for: it has to
     // advance a number of sites (a call of 2 steps at 32^3: 40 us against 35, of 4
-    // at 64^3: 56 against 58, of 2 at 80^3: 55 against 56), on columns that fill an
-    // eighth of a block of 28 x 8 (4 x 4 x 16384, 20 steps: 1089 us against 763;
-    // 4 x 200 x 200: 427 against 519).
-    if (L.ncomp == 1) {
-        const long long tiles = (long long)((L.nx + 27) / 28) * ((L.ny + 7) / 8);
-        m.on = m.on && (nsteps - 1) * L.N >= 3ll << 18 && 8ll * L.nx * L.ny >= tiles * 28 * 8;
-    }
+    // at 64^3: 56 against 58, of 2 at 80^3: 55 against 56).
+    if (L.ncomp == 1) m.on = m.on && (nsteps - 1) * L.N >= 3ll << 18;
     const size_t c = compute_bytes(ctx->prec);
     const size_t rho = align_up((size_t)L.ncomp * L.N * c), all = rho + align_up((size_t)3 * L.pstride * c);
     char* cur = (char*)L.f_cur;

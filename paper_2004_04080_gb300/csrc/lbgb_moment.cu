@@ -985,14 +985,17 @@ static int moment_chunk(const Lattice& L, long long tiles, int per_sm) {
     const long long R = (long long)device_sms() * per_sm;
     int best = L.nz;
     long long cost = -1;
-    for (int n = 1; n <= L.nz; n++) {
-        const int zc = (L.nz + n - 1) / n;
-        const long long B = tiles * ((L.nz + zc - 1) / zc), c = ((B + R - 1) / R) * (zc + 4);
+    // (each chunk once: a long lattice has as many numbers of chunks as planes, and
+    // the host would look through all of them in every step)
+    for (int zc = L.nz;;) {
+        const long long n = (L.nz + zc - 1) / zc, c = ((tiles * n + R - 1) / R) * (zc + 4);
         if (cost < 0 || c < cost) {
             cost = c;
             best = zc;
         }
         if (zc <= 2) break;
+        const int m = (L.nz + zc - 2) / (zc - 1);  // chunks of fewer planes than zc
+        zc = (L.nz + m - 1) / m;
     }
     return best;
 }

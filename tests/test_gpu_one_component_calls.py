@@ -23,9 +23,9 @@ def lattice(shape, prec):
 
 
 @pytest.mark.parametrize("prec", ["fp32", "fp16"])
-@pytest.mark.parametrize("shape,steps", [((32, 32, 32), 2), ((36, 16, 16), 20), ((4, 4, 2048), 30), ((64, 64, 64), 3)])
+@pytest.mark.parametrize("shape,steps", [((32, 32, 32), 2), ((36, 16, 16), 20), ((4, 4, 512), 30), ((64, 64, 64), 3)])
 def test_small_calls_keep_populations(shape, steps, prec):
-    assert (steps - 1) * np.prod(shape) < ENOUGH or shape[0] * shape[1] < 28
+    assert (steps - 1) * np.prod(shape) < ENOUGH
     g, o = lattice(shape, prec), lattice(shape, prec)
     g.step(steps)
     for _ in range(steps):
@@ -34,7 +34,7 @@ def test_small_calls_keep_populations(shape, steps, prec):
 
 
 @pytest.mark.parametrize("prec,tol", [("fp32", 1e-5), ("fp16", 1e-3)])
-@pytest.mark.parametrize("shape", [(4, 8, 450), (28, 9, 70), (32, 8, 66), (36, 12, 43), (60, 17, 18), (56, 33, 9)])
+@pytest.mark.parametrize("shape", [(4, 9, 400), (28, 9, 70), (32, 8, 66), (36, 12, 43), (60, 17, 18), (56, 33, 9)])
 def test_large_calls(shape, prec, tol):
     """As test_gpu_single's runs: walls, a body force, a random velocity."""
     steps = 60
