@@ -702,10 +702,9 @@ int lb_step(lb_ctx* ctx, int nsteps) {
     return LB_OK;
 }
 
-// density, wetting and wall fields of the current state (no particle terms)
-// the virtual densities find the frontier nodes by the link classes: rebuild
-// them if the node map changed outside lb_step (number of launches)
-
+// Density, wetting and wall fields of the current state (no particle terms).
+// The virtual densities find the frontier nodes by the link classes, which are
+// rebuilt first if the node map changed outside lb_step.
 static int current_forces(lb_ctx* ctx) {
     Lattice& L = ctx->L;
     if (L.ncomp == 1) return LB_OK;  // no Shan-Chen or particle terms

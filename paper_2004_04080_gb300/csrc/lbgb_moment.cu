@@ -27,9 +27,9 @@
 //   f*_i = w_i (P + q (c.h) + q),  q = 2 rho c.h,  P = rho (1 - 2/3 h.h),
 // in units of 1/36 (weights 12, 2, 1); the sums are scaled at the end.
 //
-// What bounds it: instruction issue (59 % active) and the shared-memory and
-// shuffle pipe (64 %), 488 warp instructions per two rows and plane; its 44
-// bytes a site run at 0.33 of the copy bandwidth.  The two sites of a lane
+// What bounds it: instruction issue (60 % active) and the shared-memory and
+// shuffle pipe (64 %), some 490 warp instructions per two rows and plane; its 44
+// bytes a site (DRAM sees 46) run at 0.33 of the copy bandwidth.  The two sites of a lane
 // share loop, address and exchange work, and pack without regrouping (the
 // components of one site would need their sum A + B unpacked for j): one
 // site a lane took 790 instructions per 32 sites and plane.  Everything a
