@@ -110,13 +110,14 @@ Layout layout(int nx, int ny, int nz, int prec, int maxc, int ncomp) {
     // elements) each, SKEW of padding at both ends (pop_index, pop1_index)
     l.pstride = (N + 2 * SKEW + 63) / 64 * 64;
     size_t off = 0;
-    size_t fb = (size_t)ncomp * Q * l.pstride * storage_bytes(prec);
+    // the population buffer that is free doubles as the FP64 staging area of the
+    // initial fields and the read-out (5 doubles per site), and after an odd
+    // number of steps that is the first one: both are at least that large
+    const size_t pops = (size_t)ncomp * Q * l.pstride * storage_bytes(prec), staged = (size_t)5 * N * 8;
+    const size_t fb = pops > staged ? pops : staged;
     const long long Np = ncomp == 2 ? N : 0;  // per-site arrays of the coupled lattice
-    // the second population buffer doubles as the FP64 staging area of the
-    // read-out calls (5 doubles per site), so it is at least that large
-    size_t fb1 = fb > (size_t)5 * N * 8 ? fb : (size_t)5 * N * 8;
     l.f0 = off; off = align_up(off + fb);
-    l.f1 = off; off = align_up(off + fb1);
+    l.f1 = off; off = align_up(off + fb);
     l.mom = off; off = align_up(off + (size_t)3 * (ncomp == 2 ? l.pstride : 0) * compute_bytes(prec));
     l.psi = off; off = align_up(off + (size_t)2 * Np * compute_bytes(prec));
     l.psi_wall = off; off = align_up(off + (size_t)4 * nx * ny * compute_bytes(prec));
