@@ -452,9 +452,6 @@ __global__ void __launch_bounds__(MNT, NK == 1 ? 4 : 3)
     // and -1
     const int nw = (H + 1) / 2;
     if (PART && threadIdx.x == 0) sh.count = 0;
-    const bool plain = L.spread[L.turn];
-    if (threadIdx.x < NK) sh.ref[threadIdx.x] = plain ? 0.f : L.rref[threadIdx.x];
-    if (threadIdx.x == 0 && (blockIdx.x | blockIdx.y | blockIdx.z) == 0) L.spread[L.turn == 0 ? 2 : L.turn - 1] = 0;
     // psi of the planes z0 - 2 .. z0 and the other arrays of plane z0 - 1; the
     // slots go round with the planes
     PlaneCopy<NK, PART> copy;
@@ -462,6 +459,9 @@ __global__ void __launch_bounds__(MNT, NK == 1 ? 4 : 3)
     for (int q = 0; q < 3; q++) copy.psi(L, sh, z0 - 2 + q, q);
     copy.others(L, sh, z0 - 1, 2);
     cp_async_commit();
+    // (while the copies are under way)
+    if (threadIdx.x < NK) sh.ref[threadIdx.x] = L.spread[L.turn] ? 0.f : L.rref[threadIdx.x];
+    if (threadIdx.x == 0 && (blockIdx.x | blockIdx.y | blockIdx.z) == 0) L.spread[L.turn == 0 ? 2 : L.turn - 1] = 0;
     cp_async_wait_all();
     block_barrier();
     if (warp == MW) {
@@ -735,7 +735,7 @@ __global__ void __launch_bounds__(MNT, NK == 1 ? 4 : 3)
     }
     if constexpr (PART) {
         block_barrier();
-        if (threadIdx.x == 0) list.count[blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z)] = sh.count | (plain ? LIST_PLAIN : 0);
+        if (threadIdx.x == 0) list.count[blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z)] = sh.count | (L.spread[L.turn] ? LIST_PLAIN : 0);
     }
 }
 
