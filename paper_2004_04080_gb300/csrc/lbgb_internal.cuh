@@ -676,7 +676,7 @@ __device__ __forceinline__ double acc_value(const Lattice& L, const unsigned lon
     return (double)(long long)a[0] * 5.9604644775390625e-08 + (double)a[1] * 5.421010862427522e-20;
 }
 
-// a density below L.rlow was met
+// a density below L.rlow was met (every writer of a step stores the same value)
 __device__ __forceinline__ void note_spread(const Lattice& L, int turn) {
     if (L.spread[turn] == 0) L.spread[turn] = 1;
 }
